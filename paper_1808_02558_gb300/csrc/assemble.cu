@@ -652,8 +652,8 @@ static void assemble(qp_ctx* c, const qp_scene* s, qp_contacts* out) {
   QP_CUDA(cudaGetLastError());
   QP_CUDA(cudaStreamSynchronize(st));
   c->have_contacts = true;
-  c->part_G = 0;  // the Krylov partition follows the contact set
-  c->apart_G = 0;  // and so does the fused apply's
+  c->apart_G = 0;   // the standalone apply's partition follows the contact set
+  c->cgr_chunk = 0;  // and so does the resident solver's plan
 
   out->M = M;
   out->Nc = Nc;

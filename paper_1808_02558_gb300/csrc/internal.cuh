@@ -51,7 +51,9 @@ struct DevCtl {
   double scal[16];         // scalars handed between kernels (eta, t, s, norms, ...)
 };
 
-enum Scal { S_ETA = 0, S_T, S_RDUAL, S_RT, S_S, S_RELRES, S_BNORM, S_SMAX, S_RCENT };
+enum Scal { S_ETA = 0, S_T, S_RDUAL, S_RT, S_S, S_RELRES, S_BNORM, S_SMAX, S_RCENT, S_TAGS };
+
+constexpr int CGR_NO_ROOM = 3;  // k_cg_resident: a block's bodies do not fit its shared memory
 
 struct QTTCore;
 
@@ -99,13 +101,14 @@ struct qp_ctx {
 
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   qp_qtt* last_inv = nullptr;  // last QTT inverse built by pdip_step (warm start of the next)
-  // contact partition of the fused Krylov kernel (one contiguous chunk per block)
-  int part_G = 0, part_chunk = 0, part_maxb = 0, part_nbmax = 0;
-  qp::Buf part_nb, part_bodies, part_cl;
   // contact partition of the standalone fused apply (newton_apply)
   int apart_G = 0, apart_chunk = 0, apart_maxb = 0, apart_nbmax = 0;
   qp::Buf apart_nb, apart_bodies, apart_cl;
-  qp::Buf fused_pool;
+  // exchange slots of the register-resident CG and the next solve's first tag (0: clear the slots first)
+  qp::Buf cgr_buf;
+  qp::Buf cgr_plan;    // its plan for the contact set, made for blocks of cgr_chunk contacts (0: none)
+  int cgr_chunk = 0;
+  unsigned cgr_epoch = 0, cgr_last = 0;
   qp::Buf mp_act, mp_w, mp_grad, mp_sum;  // learned warm start: activations, BF16 weights, scratch
   qp::Buf batch64, batch32, batch_table;  // batched solves: per-scene vectors; table (first context)
   qp::Buf batch_qw, tune_buf;  // batched QTT work buffers; tile-shape probe data
@@ -143,6 +146,9 @@ void sync(qp_ctx* c);
 void launch_schur_blocks(qp_ctx* c, const double* gamma, const double* lambda);
 void launch_apply64(qp_ctx* c, const double* x, double* y, bool with_H);
 void launch_apply32(qp_ctx* c, const float* x, float* y, bool with_H);
+// Jacobi-CG with the system in registers and shared memory (cg_resident.cu); false: it does not fit
+bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, double inner_tol, int maxit,
+                        int max_outer, bool mixed);
 void launch_qtt_apply(qp_ctx* c, qp_qtt* A, const void* x, void* y, qp_dtype core_dt, qp_dtype vec_dt);
 // tensor-core QTT step (qtt_tc.cu): FP32 vectors, cores with r_{k-1}, r_k <= 64;
 // in the automatic mode only BF16 cores with r_{k-1} r_k >= QTT_TC_MIN_RR
