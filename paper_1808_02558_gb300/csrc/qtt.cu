@@ -1,9 +1,11 @@
 // QTT matrices: storage, mat-vec (Sec. 3.2), and the C-ABI glue for rounding,
 // compression and inversion (implemented in qtt_linalg.cu).
+#include <algorithm>
 #include <cstring>
 
 #include "internal.cuh"
 #include "qtt_dev.cuh"
+#include "qtt_tile.cuh"
 
 namespace qp {
 namespace {
@@ -24,6 +26,77 @@ template <class TV, class TA, class TC>
 __global__ void __launch_bounds__(256, 2) k_qtt_step2(QttDev q, int k, const TV* in, TV* out, int bound) {
   __shared__ Quad<TA> gq[QTT_GQ];
   qtt_step2_grid<TV, TA, TC>(q, k, in, out, gq, bound);
+}
+
+// A pass of m cores in shared memory (qtt_tile.cuh).
+template <int R, class TC>
+__global__ void __launch_bounds__(QT_THREADS, R <= 12 ? 2 : 1)
+    k_qtt_tile(const __grid_constant__ QttDev q, int k, int m, const float* __restrict__ in, float* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char qt_smem[];
+  tile_pass<R, TC>(q, k, m, in, out, qt_smem, blockIdx.x, gridDim.x);
+}
+
+template <int R, class TC>
+void launch_tile(qp_ctx* c, const QttDev& q, int k, int m, const float* in, float* out) {
+  auto kern = k_qtt_tile<R, TC>;
+  const int smem = tile_bytes(R, m);
+  QP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_bytes(R, QT_MAXM)));
+  const long long ntiles = (1LL << (q.d - m)) / QT_NC;
+  kern<<<(int)std::min<long long>(ntiles, 2 * c->num_sms), QT_THREADS, smem, c->stream>>>(q, k, m, in, out);
+}
+
+template <class TC>
+void launch_tile_r(qp_ctx* c, const QttDev& q, int k, int m, int R, const float* in, float* out) {
+  if (R == 4) launch_tile<4, TC>(c, q, k, m, in, out);
+  else if (R == 8) launch_tile<8, TC>(c, q, k, m, in, out);
+  else if (R == 10) launch_tile<10, TC>(c, q, k, m, in, out);
+  else if (R == 12) launch_tile<12, TC>(c, q, k, m, in, out);
+  else launch_tile<16, TC>(c, q, k, m, in, out);
+}
+
+// FP64 step, bound by the FP64 pipe (two multiply-adds a clock and SM) or, at small
+// sizes, by its 64-cycle latency: a column item's output ranks are spread over
+// `split` threads (consecutive items on consecutive lanes), so that 2^12 values at
+// rank 10 fill the chip -- a thread an item left 148 SMs idle and 400 dependent
+// multiply-adds a thread: 67 us a core, this 6.
+__global__ void __launch_bounds__(256)
+    k_qtt_step64(const __grid_constant__ QttDev q, int k, const double* __restrict__ in, double* __restrict__ out,
+                 long long items, int split) {
+  const int r0 = q.ranks[k - 1], r1 = q.ranks[k], lowbits = q.d - k;
+  const long long nI = 1LL << lowbits;
+  const double* G = static_cast<const double*>(q.cores) + q.off[k - 1];
+  const long long n = items * split;
+  for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < n; w += (long long)gridDim.x * blockDim.x) {
+    const int part = (int)(w >> (q.d - 1));  // items = 2^(d-1)
+    const long long it = w & (items - 1);
+    const long long I = it & (nI - 1), Jp = it >> lowbits;
+    const double* in0 = in + ((2 * Jp) * r1 << lowbits) + I;
+    const double* in1 = in0 + ((long long)r1 << lowbits);
+    double* o = out + ((Jp * r0) << (lowbits + 1)) + I;
+    for (int a = part; a < r0; a += split) {
+      const double* Ga = G + (long long)a * 4 * r1;
+      double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
+#pragma unroll 10
+      for (int b = 0; b < r1; ++b) {
+        const double v0 = __ldg(in0 + ((long long)b << lowbits)), v1 = __ldg(in1 + ((long long)b << lowbits));
+        p0 = fma(__ldg(Ga + b), v0, p0);
+        p1 = fma(__ldg(Ga + r1 + b), v1, p1);
+        q0 = fma(__ldg(Ga + 2 * r1 + b), v0, q0);
+        q1 = fma(__ldg(Ga + 3 * r1 + b), v1, q1);
+      }
+      o[(long long)a << (lowbits + 1)] = p0 + p1;
+      o[((long long)a << (lowbits + 1)) + nI] = q0 + q1;
+    }
+  }
+}
+
+void launch_step64(qp_ctx* c, const QttDev& q, int k, const double* in, double* out) {
+  const long long items = 1LL << (q.d - 1);
+  // at least 512 threads an SM, while there are output ranks to spread
+  const long long want = (long long)c->num_sms * 512;
+  const int split = (int)std::max<long long>(1, std::min<long long>(q.ranks[k - 1], (want + items - 1) / items));
+  const long long blocks = std::min<long long>((items * split + 255) / 256, (long long)c->num_sms * 8);
+  k_qtt_step64<<<(int)blocks, 256, 0, c->stream>>>(q, k, in, out, items, split);
 }
 
 template <class TV, class TA, class TC>
@@ -141,14 +214,22 @@ void launch_qtt_apply(qp_ctx* c, qp_qtt* A, const void* x, void* y, qp_dtype cdt
   bool used_tc = false;
   for (int k = A->d; k >= 1; ++pass) {
     const bool tcs = tc_ok && qtt_tc_eligible(c, q, k, cdt);
-    const int bound = (vdt == QP_F64 || tcs || tc_all) ? 0 : qtt_fuse_bound<float>(q, k, QTT_GQ);
-    const int next = bound ? k - 2 : k - 1;
+    int R = 0;
+    const int tile = (vdt == QP_F64 || tcs || tc_all) ? 0 : tile_plan(q, k, R);
+    const int bound = (vdt == QP_F64 || tcs || tc_all || tile) ? 0 : qtt_fuse_bound<float>(q, k, QTT_GQ);
+    const int next = tile ? k - tile : (bound ? k - 2 : k - 1);
     void* out = (next == 0) ? y : ((pass & 1) ? w1 : w0);
     if (tcs) {
       if (!used_tc) QP_CUDA(cudaMemsetAsync(qtt_tc_flag(c), 0, sizeof(int), c->stream));
       used_tc = true;
       launch_qtt_step_tc(c, q, k, static_cast<const float*>(in), static_cast<float*>(out), cdt);
-    } else if (vdt == QP_F64) launch_step<double, double, double>(c, q, k, in, out, bound, N);
+    } else if (tile) {
+      const float* fi = static_cast<const float*>(in);
+      float* fo = static_cast<float*>(out);
+      if (cdt == QP_F32) launch_tile_r<float>(c, q, k, tile, R, fi, fo);
+      else if (cdt == QP_BF16) launch_tile_r<__nv_bfloat16>(c, q, k, tile, R, fi, fo);
+      else launch_tile_r<double>(c, q, k, tile, R, fi, fo);
+    } else if (vdt == QP_F64) launch_step64(c, q, k, static_cast<const double*>(in), static_cast<double*>(out));
     else if (cdt == QP_F32) launch_step<float, float, float>(c, q, k, in, out, bound, N);
     else if (cdt == QP_BF16) launch_step<float, float, __nv_bfloat16>(c, q, k, in, out, bound, N);
     else launch_step<float, float, double>(c, q, k, in, out, bound, N);
