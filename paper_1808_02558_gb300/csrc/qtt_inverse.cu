@@ -30,7 +30,9 @@ __device__ inline double blk_sum(double v) { return dla::block_sum(v); }
 extern __shared__ double la_smem[];
 
 __device__ inline void blk_syev(double* A, double* V, double* Vs, double* w, int n) {
-  dla::syev(A, V, Vs, w, n, la_smem);
+  // no FP32 start: the sweeps over the cores amplify any change of the factors, and most
+  // of their orders are beyond its range
+  dla::syev(A, V, Vs, w, n, la_smem, false);
 }
 
 struct DmrgArgs {

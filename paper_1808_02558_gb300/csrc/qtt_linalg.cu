@@ -31,8 +31,8 @@ __device__ inline double cta_sum(double v) { return dla::block_sum(v); }
 // dynamic shared memory of the one-block kernels (the eigensolver's staging area)
 extern __shared__ double la_smem[];
 
-__device__ inline void cta_syev(double* A, double* V, double* Vs, double* w, int n) {
-  dla::syev(A, V, Vs, w, n, la_smem);
+__device__ inline void cta_syev(double* A, double* V, double* Vs, double* w, int n, bool f32) {
+  dla::syev(A, V, Vs, w, n, la_smem, f32);
 }
 
 // ---------------------------------------------------------------- rounding
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(LT) k_tt_round(RoundArgs a) {
       a.A[i] = s;
     }
     __syncthreads();
-    cta_syev(a.A, a.V, a.Vs, a.w, rk);
+    cta_syev(a.A, a.V, a.Vs, a.w, rk, false);  // divides by the root of small eigenvalues
     if (tid == 0) {
       double lmax = fmax(a.w[0], 0.0);
       int r = 0;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(LT) k_tt_round(RoundArgs a) {
       a.A[i] = s;
     }
     __syncthreads();
-    cta_syev(a.A, a.V, a.Vs, a.w, rn);
+    cta_syev(a.A, a.V, a.Vs, a.w, rn, false);
     if (tid == 0) sh_r = trunc_rank(a.w, rn, delta, a.rmax);
     __syncthreads();
     const int r = sh_r;
@@ -468,10 +468,11 @@ struct EigArgs {
   double delta;
   int rmax;
   int* rank_out;
+  bool f32;  // the FP32 start may be taken
 };
 
 __global__ void __launch_bounds__(LT) k_eig_trunc(EigArgs e) {
-  cta_syev(e.A, e.V, e.Vs, e.w, e.n);
+  cta_syev(e.A, e.V, e.Vs, e.w, e.n, e.f32);
   if (threadIdx.x == 0) *e.rank_out = trunc_rank(e.w, e.n, e.delta, e.rmax);
 }
 
@@ -871,6 +872,7 @@ qp_qtt* compress_impl(qp_ctx* c, bool with_H, double eps, int rmax, const double
     ea.rmax = rmax;
     int* rk_dev = reinterpret_cast<int*>(static_cast<double*>(w.tmp.p) + 512);
     ea.rank_out = rk_dev;
+    ea.f32 = eps >= dla::SYEV_F32_EPS;
     if (n <= dla::SYEV_SMEM_N) {
       QP_CUDA(cudaFuncSetAttribute(k_eig_trunc, cudaFuncAttributeMaxDynamicSharedMemorySize, dla::SYEV_SMEM_BYTES));
       k_eig_trunc<<<1, LT, dla::SYEV_SMEM_BYTES, st>>>(ea);
