@@ -120,7 +120,7 @@ int qp_destroy(qp_ctx_t c) {
   Buf* bufs[] = {&c->ca, &c->cb, &c->phi, &c->frame, &c->point, &c->arm_a, &c->arm_b, &c->key, &c->r,
                  &c->rec64, &c->rec32, &c->inv_m, &c->inv_I, &c->inv_m32, &c->inv_I32,
                  &c->bptr, &c->inc, &c->wbody, &c->wbody32, &c->H, &c->H32, &c->dinv, &c->dinv32,
-                 &c->partial, &c->ctl, &c->cgr_buf, &c->cgr_plan, &c->batch64, &c->batch32,
+                 &c->partial, &c->ctl, &c->cgr_buf, &c->cmp_start, &c->cgr_plan, &c->batch64, &c->batch32,
                  &c->batch_table, &c->mp_act, &c->mp_w, &c->mp_grad, &c->mp_sum};
   for (Buf* b : bufs) b->release();
   for (auto& b : c->v64) b.release();

@@ -95,6 +95,7 @@ struct qp_ctx {
   qp::Buf partial;     // per-block partial sums
   qp::Buf ctl;         // DevCtl
   qp::Buf scratch[8];  // assembly / QTT scratch
+  qp::Buf cmp_start;   // compression: the parents' first child rows, children, order by children
   qp::Buf la[6];       // one-block linear algebra workspaces (A, V, Vs, w, tmp, misc)
   qp::Buf dm[16];      // QTT inverse workspaces
   qp::DevCtl* ctl_host = nullptr;  // pinned mirror

@@ -354,15 +354,40 @@ __global__ void k_parent_flags(long long n, const unsigned long long* __restrict
     flag[i] = (i == 0 || (key[i] >> 2) != (key[i - 1] >> 2)) ? 1 : 0;
 }
 
-// M[pid, child*r + a] = W[i, a];  parent key list
+// First child row of each parent (its child rows are consecutive, in the order of their
+// digits), the set of its children as a mask, its index, and its key.
+__global__ void k_parents(long long n, const unsigned long long* __restrict__ key, const int* __restrict__ pid,
+                          int* __restrict__ start, unsigned char* __restrict__ mask, int* __restrict__ index,
+                          unsigned long long* __restrict__ pkey) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const unsigned long long k = key[i] >> 2;
+    if (i == 0 || k != (key[i - 1] >> 2)) {
+      const int p = pid[i] - 1;
+      unsigned m = 0;
+      for (long long j = i; j < n && j < i + 4 && (key[j] >> 2) == k; ++j) m |= 1u << (key[j] & 3ull);
+      start[p] = (int)i;
+      mask[p] = (unsigned char)m;
+      index[p] = p;
+      pkey[p] = k;
+    }
+  }
+}
+
+// off[m] = number of sorted masks below m, m = 0..16.
+__global__ void k_mask_bounds(int n, const unsigned char* __restrict__ mask, int* __restrict__ off) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x) {
+    const int lo = i == 0 ? 0 : mask[i - 1] + 1, hi = i == n ? 16 : mask[i];
+    for (int m = lo; m <= hi; ++m) off[m] = i;
+  }
+}
+
+// M[pid, child*r + a] = W[i, a] (zero elsewhere; only ranks above 16 need M itself)
 __global__ void k_scatter_rows(long long n, int r, const unsigned long long* __restrict__ key,
-                               const int* __restrict__ pid, const double* __restrict__ W, double* __restrict__ Mx,
-                               unsigned long long* __restrict__ pkey) {
+                               const int* __restrict__ pid, const double* __restrict__ W, double* __restrict__ Mx) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int p = pid[i] - 1;
     const int ch = (int)(key[i] & 3ull);
     for (int a = 0; a < r; ++a) Mx[(long long)p * 4 * r + ch * r + a] = W[i * r + a];
-    if (i == 0 || (key[i] >> 2) != (key[i - 1] >> 2)) pkey[p] = key[i] >> 2;
   }
 }
 
@@ -380,20 +405,65 @@ __global__ void k_gram_partial(long long rows, int n, const double* __restrict__
   }
 }
 
-// The same partial Gram matrices for n = 4 r <= 64, register-tiled: the block
-// stages GR_ROWS rows of its chunk in shared memory, thread t owns the 4 x 4
-// tile (tx, ty), tx <= ty, of the upper triangle in row group g (groups take
-// every G-th staged row, so all 256 threads work at small n); the groups' tiles
-// are then added in group order into the block's partial (both triangles).
-// Partials are summed in block order by k_gram_reduce: the result does not
-// depend on scheduling.  Dynamic shared memory: GR_SMEM bytes.
-constexpr int GR_ROWS = 64;
-constexpr int GR_SMEM = 60 * 1024;  // >= GR_ROWS * 64 doubles and >= G n^2 doubles for every n = 4 r <= 64
-__global__ void __launch_bounds__(256) k_gram_tiled(long long rows, int n, const double* __restrict__ Mx,
-                                                    double* __restrict__ part, long long chunk) {
-  extern __shared__ double gr_sm[];
-  const int T = n >> 2, ntiles = T * (T + 1) / 2;
-  const int G = 256 / ntiles;  // row groups (>= 1 for n <= 64)
+// Gram matrices for ranks to 16 (n = 4 r <= 64) by the sets of children: on average two
+// or three of a parent's four children exist, and M's rows are zero elsewhere.  The
+// parents are sorted by mask; a block takes a run of parents of one mask with m children,
+// whose rows of M without the zeros are the m r consecutive entries of W from the first
+// child on, and forms their Gram matrix of order m r: a quarter to a third of the FP64
+// multiplications, which bound this.  A 2^20 compression of rank 10 spends 2.8 ms here,
+// sorting included; the dense rows took 6.3 and their clearing and scattering 1.9.
+struct MaskTable {
+  int off[17];    // parents of each mask in the sorted order
+  int first[17];  // first block of each mask
+  int chunk[16];  // parents per block
+};
+
+// Blocks over the masks by cost (4 x 4 tiles per row), at most nblk + 15 of them.  All
+// threads of the block call it.
+__device__ inline void mask_table(const int* __restrict__ off, int r, int nblk, MaskTable& t) {
+  const int m = threadIdx.x;
+  if (m < 32) {
+    const int T = (__popc(m & 15) * r + 3) >> 2, cost = T * (T + 1) / 2 + T;
+    const int o = off[min(m, 16)], cnt = m >= 1 && m < 16 ? off[m + 1] - o : 0;
+    long long total = (long long)cnt * cost;
+    for (int k = 16; k > 0; k >>= 1) total += __shfl_xor_sync(~0u, total, k);
+    const long long per = (total + nblk - 1) / nblk;
+    const int chunk = cnt > 0 ? (int)((per + cost - 1) / cost) : 1;
+    const int blocks = (cnt + chunk - 1) / chunk;
+    int before = blocks;
+    for (int k = 1; k < 32; k <<= 1) {
+      const int v = __shfl_up_sync(~0u, before, k);
+      if (m >= k) before += v;
+    }
+    if (m <= 16) {
+      t.off[m] = o;
+      t.first[m] = before - blocks;
+    }
+    if (m < 16) t.chunk[m] = chunk;
+  }
+  __syncthreads();
+}
+
+// Thread t owns the 4 x 4 tile (tx, ty), tx <= ty, of the upper triangle in row group g
+// (groups take every G-th staged row, so all 256 threads work at small orders); the
+// groups' tiles are added in group order into the block's partial, m r square in n x n.
+// k_gram_reduce adds the partials in block order: the result does not depend on
+// scheduling.  Dynamic shared memory: GR_SMEM bytes.
+constexpr int GR_ROWS = 128;
+constexpr int GR_SMEM = 60 * 1024;  // >= 64 rows of 64 doubles and >= G l^2 doubles for every l = 4 T <= 64
+__global__ void __launch_bounds__(256, 3)
+    k_gram_masks(int r, int nblk, const double* __restrict__ W, const int* __restrict__ start,
+                 const int* __restrict__ index, const int* __restrict__ off, double* __restrict__ part) {
+  extern __shared__ __align__(16) double gr_sm[];
+  __shared__ MaskTable tab;
+  __shared__ int row0[GR_ROWS];
+  mask_table(off, r, nblk, tab);
+  const int b = blockIdx.x;
+  if (b >= tab.first[16]) return;
+  int m = 1;
+  while (m < 15 && b >= tab.first[m + 1]) ++m;
+  const int nc = __popc(m) * r, T = (nc + 3) >> 2, ld = 4 * T, ntiles = T * (T + 1) / 2;
+  const int G = 256 / ntiles;  // row groups (>= 1: ntiles <= 136)
   const int tid = threadIdx.x, g = tid / ntiles, tile = tid - g * ntiles;
   const bool active = g < G;
   int tx = 0, ty = 0;
@@ -405,56 +475,135 @@ __global__ void __launch_bounds__(256) k_gram_tiled(long long rows, int n, const
     }
     tx = rem;  // 0 <= tx <= ty
   }
+  const int cap = min(GR_ROWS, GR_SMEM / 8 / ld);
+  const int r0 = tab.off[m] + (b - tab.first[m]) * tab.chunk[m], r1 = min(tab.off[m + 1], r0 + tab.chunk[m]);
   double acc[4][4] = {};
-  const long long r0 = blockIdx.x * chunk;
-  const long long r1 = min(rows, r0 + chunk);
-  for (long long base = r0; base < r1; base += GR_ROWS) {
-    const int nr = (int)min((long long)GR_ROWS, r1 - base);
+  for (int base = r0; base < r1; base += cap) {
+    const int nr = min(cap, r1 - base);
     __syncthreads();
-    for (int i = tid; i < nr * n; i += 256) gr_sm[i] = Mx[base * n + i];
+    if (tid < nr) row0[tid] = __ldg(start + __ldg(index + base + tid));
+    __syncthreads();
+    for (int i = tid; i < nr * ld; i += 256) {
+      const int row = i / ld, a = i - row * ld;
+      gr_sm[i] = a < nc ? __ldg(W + (long long)row0[row] * r + a) : 0.0;
+    }
     __syncthreads();
     if (active) {
       for (int rr = g; rr < nr; rr += G) {
-        const double* row = gr_sm + rr * n;
-        double a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          a[i] = row[4 * tx + i];
-          b[i] = row[4 * ty + i];
-        }
+        const double2* row = reinterpret_cast<const double2*>(gr_sm + rr * ld);
+        const double2 a0 = row[2 * tx], a1 = row[2 * tx + 1], b0 = row[2 * ty], b1 = row[2 * ty + 1];
+        const double a[4] = {a0.x, a0.y, a1.x, a1.y}, bb[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
       }
     }
   }
   __syncthreads();
-  const int nn = n * n;
+  const int ll = ld * ld;
   if (active) {
-    double* red = gr_sm + g * nn;
+    double* red = gr_sm + g * ll;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int x = 4 * tx + i, y = 4 * ty + j;
-        red[x * n + y] = acc[i][j];
-        red[y * n + x] = acc[i][j];
+        red[x * ld + y] = acc[i][j];
+        red[y * ld + x] = acc[i][j];
       }
   }
   __syncthreads();
-  double* out = part + (long long)blockIdx.x * nn;
-  for (int xy = tid; xy < nn; xy += 256) {
-    double v = 0.0;
-    for (int q = 0; q < G; ++q) v += gr_sm[q * nn + xy];
-    out[xy] = v;
+  double* out = part + (long long)b * 16 * r * r;
+  for (int i = tid; i < ll; i += 256) {
+    const int x = i / ld, y = i - x * ld;
+    if (x >= nc || y >= nc) continue;
+    double sum = 0.0;
+    for (int q = 0; q < G; ++q) sum += gr_sm[q * ll + i];
+    out[x * nc + y] = sum;
   }
 }
 
-__global__ void k_gram_reduce(int nparts, int n, const double* __restrict__ part, double* __restrict__ G) {
-  for (int xy = blockIdx.x * blockDim.x + threadIdx.x; xy < n * n; xy += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int p = 0; p < nparts; ++p) s += part[(long long)p * n * n + xy];
+// G = sum of the partials of the masks that hold both children, in block order: a block
+// takes 32 entries, its 16 warps a share of the partials each, added in warp order.
+__global__ void __launch_bounds__(512) k_gram_reduce_masks(int r, int nblk, const int* __restrict__ off,
+                                                           const double* __restrict__ part, double* __restrict__ G) {
+  __shared__ MaskTable tab;
+  __shared__ double sm[16][33];
+  mask_table(off, r, nblk, tab);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = 4 * r;
+  const int xy = blockIdx.x * 32 + lane;
+  const int q0 = tab.first[16] * w / 16, q1 = tab.first[16] * (w + 1) / 16;
+  double s = 0.0;
+  if (xy < n * n) {
+    const int x = xy / n, y = xy - x * n, c = x / r, d = y / r;
+    for (int m = 1; m < 16; ++m) {
+      if (!((m >> c) & 1) || !((m >> d) & 1)) continue;
+      const int nc = __popc(m) * r, at = (__popc(m & ((1 << c) - 1)) * r + x - c * r) * nc +
+                                         __popc(m & ((1 << d) - 1)) * r + y - d * r;
+      const int e = min(q1, tab.first[m + 1]);
+#pragma unroll 4
+      for (int q = max(q0, tab.first[m]); q < e; ++q) s += __ldg(part + (long long)q * n * n + at);
+    }
+  }
+  sm[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && xy < n * n) {
+    s = 0.0;
+    for (int q = 0; q < 16; ++q) s += sm[q][lane];
+    G[xy] = s;
+  }
+}
+
+// Partial 4 x 4 Gram matrices of the first level (rank 1): a thread a parent.
+__global__ void __launch_bounds__(256) k_gram_first(int rows, const double* __restrict__ W,
+                                                    const unsigned char* __restrict__ mask,
+                                                    const int* __restrict__ start, double* __restrict__ part) {
+  double acc[10] = {};
+  for (int p = blockIdx.x * 256 + threadIdx.x; p < rows; p += gridDim.x * 256) {
+    const unsigned m = mask[p];
+    const double* w = W + start[p];
+    double v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = (m >> c) & 1u ? __ldg(w + __popc(m & ((1u << c) - 1))) : 0.0;
+    int q = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int d = c; d < 4; ++d, ++q) acc[q] = fma(v[c], v[d], acc[q]);
+  }
+  int q = 0;
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int d = c; d < 4; ++d, ++q) {
+      const double t = cta_sum(acc[q]);
+      if (threadIdx.x == 0) {
+        part[blockIdx.x * 16 + c * 4 + d] = t;
+        part[blockIdx.x * 16 + d * 4 + c] = t;
+      }
+    }
+}
+
+// G = sum of the partials in order: a block takes 32 entries, its 16 warps a share of
+// the partials each, added in warp order (a thread an entry read them one after the
+// other: 33 us a level).
+__global__ void __launch_bounds__(512) k_gram_reduce(int nparts, int n, const double* __restrict__ part,
+                                                     double* __restrict__ G) {
+  __shared__ double sm[16][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int xy = blockIdx.x * 32 + lane;
+  const int q0 = nparts * w / 16, q1 = nparts * (w + 1) / 16;
+  double s = 0.0;
+  if (xy < n * n) {
+#pragma unroll 8
+    for (int p = q0; p < q1; ++p) s += __ldg(part + (long long)p * n * n + xy);
+  }
+  sm[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && xy < n * n) {
+    s = 0.0;
+    for (int q = 0; q < 16; ++q) s += sm[q][lane];
     G[xy] = s;
   }
 }
@@ -655,16 +804,27 @@ __global__ void k_core_from_V(int n, int r, int rnew, const double* __restrict__
   }
 }
 
-// Wn[row][a] = sum_x M[row][x] Vs[x][a]
-__global__ void k_project(long long rows, int n, int rnew, const double* __restrict__ Mx,
-                          const double* __restrict__ Vs, double* __restrict__ Wn) {
+// Wn[p][a] = sum over p's children of sum_al W[child][al] Vs[(digit r + al)][a] (what the
+// row of M times Vs is without M's zeros).  Parents come in the order of their masks, so
+// a warp's threads have the same children.  Bound by the FP64 pipe (m r rnew fused
+// multiply-adds a parent): 2.0 ms of a 2^20 compression of rank 10, 3.05 with the zeros.
+__global__ void k_project(long long rows, int r, int rnew, const double* __restrict__ W,
+                          const unsigned char* __restrict__ mask, const int* __restrict__ index,
+                          const int* __restrict__ start, const double* __restrict__ Vs, double* __restrict__ Wn) {
+  const int n = 4 * r;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < rows * rnew;
        i += (long long)gridDim.x * blockDim.x) {
-    const long long row = i / rnew;
-    const int a = (int)(i - row * rnew);
+    const int u = (int)(i / rnew);
+    const int p = __ldg(index + u), a = (int)(i - (long long)u * rnew);
+    const double* w = W + (long long)__ldg(start + p) * r;
     double s = 0.0;
-    for (int x = 0; x < n; ++x) s += Mx[row * n + x] * Vs[x * n + a];
-    Wn[i] = s;
+    for (unsigned m = __ldg(mask + u); m; m &= m - 1) {
+      const double* v = Vs + (long long)(__ffs(m) - 1) * r * n + a;
+#pragma unroll 5
+      for (int x = 0; x < r; ++x) s = fma(__ldg(w + x), __ldg(v + (long long)x * n), s);
+      w += r;
+    }
+    Wn[(long long)p * rnew + a] = s;
   }
 }
 
@@ -831,6 +991,7 @@ qp_qtt* compress_impl(qp_ctx* c, bool with_H, double eps, int rmax, const double
   Buf& b_M = c->scratch[5];
   Buf& b_W = c->scratch[6];
   Buf& b_part = c->scratch[7];
+  Buf& b_start = c->cmp_start;
   for (int k = d; k >= 2; --k) {
     int* flag = static_cast<int*>(b_flag.ensure(2 * rows * sizeof(int) + 64));
     int* pid = flag + rows;
@@ -843,25 +1004,46 @@ qp_qtt* compress_impl(qp_ctx* c, bool with_H, double eps, int rmax, const double
     QP_CUDA(cudaMemcpyAsync(&npar, pid + rows - 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     QP_CUDA(cudaStreamSynchronize(st));
     const int n = 4 * r;
-    double* Mx = static_cast<double*>(b_M.ensure((size_t)npar * n * sizeof(double)));
-    QP_CUDA(cudaMemsetAsync(Mx, 0, (size_t)npar * n * sizeof(double), st));
-    k_scatter_rows<<<c->num_sms * 8, 256, 0, st>>>(rows, r, K, pid, W, Mx, Kalt);
-    // Gram: register-tiled partials for n <= 64, one entry per thread above
+    // first rows, index, sorted index, 17 bounds; masks, sorted masks
+    const size_t np16 = ((size_t)npar + 15) / 16 * 16;
+    int* start = static_cast<int*>(b_start.ensure((3 * np16 + 32) * sizeof(int) + 2 * np16));
+    int *index = start + np16, *index_s = index + np16, *moff = index_s + np16;
+    unsigned char *mask = reinterpret_cast<unsigned char*>(moff + 32), *mask_s = mask + np16;
+    k_parents<<<c->num_sms * 8, 256, 0, st>>>(rows, K, pid, start, mask, index, Kalt);
+    QP_CUDA(cudaGetLastError());
     double* G = static_cast<double*>(w.A.ensure((size_t)n * n * sizeof(double)));
-    if (n <= 64) {
-      const int nparts = (int)std::min<long long>(2 * c->num_sms, std::max<long long>(1, npar / 256));
-      const long long chunk = (npar + nparts - 1) / nparts;
-      double* gp = static_cast<double*>(b_part.ensure((size_t)nparts * n * n * sizeof(double)));
-      QP_CUDA(cudaFuncSetAttribute(k_gram_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, GR_SMEM));
-      k_gram_tiled<<<nparts, 256, GR_SMEM, st>>>(npar, n, Mx, gp, chunk);
-      k_gram_reduce<<<ceil_div((long long)n * n, 256), 256, 0, st>>>(nparts, n, gp, G);
+    if (r >= 2) {  // the first level needs no order: its Gram matrix is a thread a parent
+      tb = 0;
+      cub::DeviceRadixSort::SortPairs(nullptr, tb, mask, mask_s, index, index_s, npar, 0, 4, st);
+      tmp = c->scratch[1].ensure(tb);
+      QP_CUDA(cub::DeviceRadixSort::SortPairs(tmp, tb, mask, mask_s, index, index_s, npar, 0, 4, st));
     } else {
+      mask_s = mask;
+      index_s = index;
+    }
+    if (r == 1) {
+      const int nparts = (int)std::min<long long>(4 * c->num_sms, ceil_div(npar, 256));
+      double* gp = static_cast<double*>(b_part.ensure((size_t)nparts * n * n * sizeof(double)));
+      k_gram_first<<<nparts, 256, 0, st>>>(npar, W, mask, start, gp);
+      k_gram_reduce<<<1, 512, 0, st>>>(nparts, n, gp, G);
+    } else if (n <= 64) {
+      const int nblk = (int)std::min<long long>(3 * c->num_sms - 15, std::max<long long>(1, npar / 128));
+      double* gp = static_cast<double*>(b_part.ensure((size_t)(nblk + 15) * n * n * sizeof(double)));
+      k_mask_bounds<<<c->num_sms * 4, 256, 0, st>>>(npar, mask_s, moff);
+      QP_CUDA(cudaFuncSetAttribute(k_gram_masks, cudaFuncAttributeMaxDynamicSharedMemorySize, GR_SMEM));
+      k_gram_masks<<<nblk + 15, 256, GR_SMEM, st>>>(r, nblk, W, start, index_s, moff, gp);
+      k_gram_reduce_masks<<<ceil_div((long long)n * n, 32), 512, 0, st>>>(r, nblk, moff, gp, G);
+    } else {
+      double* Mx = static_cast<double*>(b_M.ensure((size_t)npar * n * sizeof(double)));
+      QP_CUDA(cudaMemsetAsync(Mx, 0, (size_t)npar * n * sizeof(double), st));
+      k_scatter_rows<<<c->num_sms * 8, 256, 0, st>>>(rows, r, K, pid, W, Mx);
       const int nparts = (int)std::min<long long>(256, std::max<long long>(1, npar / 64));
       const long long chunk = (npar + nparts - 1) / nparts;
       double* gp = static_cast<double*>(b_part.ensure((size_t)nparts * n * n * sizeof(double)));
       k_gram_partial<<<nparts, 256, 0, st>>>(npar, n, Mx, gp, chunk);
-      k_gram_reduce<<<ceil_div((long long)n * n, 256), 256, 0, st>>>(nparts, n, gp, G);
+      k_gram_reduce<<<ceil_div((long long)n * n, 32), 512, 0, st>>>(nparts, n, gp, G);
     }
+    QP_CUDA(cudaGetLastError());
     EigArgs ea;
     ea.A = G;
     ea.V = static_cast<double*>(w.V.ensure((size_t)n * n * sizeof(double)));
@@ -902,18 +1084,16 @@ qp_qtt* compress_impl(qp_ctx* c, bool with_H, double eps, int rmax, const double
     // core k (1-based) -> index k-1: shape (rnew, 4, r)
     double* core = static_cast<double*>(cb_store[k - 1].ensure((size_t)rnew * n * sizeof(double)));
     k_core_from_V<<<ceil_div((long long)rnew * n, 256), 256, 0, st>>>(n, r, rnew, ea.Vs, core);
-    double* Wn = static_cast<double*>(b_W.ensure((size_t)npar * rnew * sizeof(double)));
-    k_project<<<c->num_sms * 8, 256, 0, st>>>(npar, n, rnew, Mx, ea.Vs, Wn);
+    // W and Wn in turn in two buffers (the entries' values in the first are done with)
+    Buf& b_Wn = (d - k) % 2 == 0 ? b_W : c->scratch[3];
+    double* Wn = static_cast<double*>(b_Wn.ensure((size_t)npar * rnew * sizeof(double)));
+    k_project<<<c->num_sms * 8, 256, 0, st>>>(npar, r, rnew, W, mask_s, index_s, start, ea.Vs, Wn);
     QP_CUDA(cudaGetLastError());
     // next level: rows = parents
     rows = npar;
     r = rnew;
     std::swap(K, Kalt);
-    // W must not alias the next level's M: copy into the value scratch
-    double* Wkeep = static_cast<double*>(c->scratch[3].ensure((size_t)rows * r * sizeof(double) * 2));
-    QP_CUDA(cudaMemcpyAsync(Wkeep, Wn, (size_t)rows * r * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    W = Wkeep;
-    // keys: K now points to the parent keys written by k_scatter_rows into Kalt (swapped)
+    W = Wn;
   }
   // first core (k = 1): rows <= 4 with keys b_1
   QP_REQUIRE(rows <= 4, QP_CUDA_ERROR, "qtt_compress: inconsistent top level");
