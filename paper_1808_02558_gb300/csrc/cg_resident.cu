@@ -89,6 +89,7 @@ struct CgrArgs {
   int maxit, max_outer;
   unsigned epoch;        // first tag of this solve
   double* r64;           // [P] FP64 residual
+  double* xbest;         // [P] the replaced x of the smallest true residual, while x is not it
   u64* halo;             // [2][G][CR_HALO / 2][rcap][2] inboxes, pairs of words by place
   u64* red;              // [2][CR_RED]
   DevCtl* ctl;
@@ -141,6 +142,9 @@ struct CgrShared {
   double poll[32][8];           // per warp: sums over its share of the blocks' messages
   double scal[8];                // what the sum's last step hands to the block
   int flag[2];
+  double best;                   // smallest true residual norm so far
+  double keep2;                  // squared growth of the residual up to which the direction is kept
+  int held;                      // x is the (nonzero) solution that has it
   // the block's lists (CgrPlan's, in shared memory)
   int c0, c1, chunk, nbcap, rcap, nbord, nint, nrem;
   double* wr;             // [chunk][CR_WR] wrenches of the block's contacts (viewed as T)
@@ -782,21 +786,25 @@ struct Own {
         for (int u = 0; u < 3; ++u) r[k][u] = (T)(v[row + u] * inv);
       }
   }
-  // x += scale e (and p aside, where it is not kept in registers over a residual)
+  // x += scale e, the best x aside (and p, where it is not kept in registers over a residual)
   __device__ __forceinline__ void put_x(const CgrArgs& A, CgrShared& sh, double scale) {
+    const bool held = sh.held;
 #pragma unroll
     for (int k = 0; k < KC; ++k)
       if (on(k)) {
         const int lc = t + k * NT;
-        double* x = A.x + (long long)A.s64.slots * (sh.c0 + lc);
+        const long long row = (long long)A.s64.slots * (sh.c0 + lc);
+        double* x = A.x + row;
+        const double old[3] = {x[0], x[1], x[2]};  // all loads before a store
 #pragma unroll
         for (int u = 0; u < 3; ++u) {
           if constexpr (SM) {
-            x[u] += scale * (double)es[3 * lc + u];
+            x[u] = old[u] + scale * (double)es[3 * lc + u];
             ps[3 * lc + u] = pr[k][u];
           } else {
-            x[u] += scale * (double)er[k][u];
+            x[u] = old[u] + scale * (double)er[k][u];
           }
+          if (held) A.xbest[row + u] = old[u];
         }
       }
   }
@@ -936,7 +944,9 @@ struct Rows {
   }
   __device__ __forceinline__ void put_x(const CgrArgs& A, CgrShared& sh, double scale) {
     if (act) {
-      A.x[(long long)A.s64.slots * (sh.c0 + lc) + u] += scale * (double)e;
+      const long long row = (long long)A.s64.slots * (sh.c0 + lc) + u;
+      if (sh.held) A.xbest[row] = A.x[row];
+      A.x[row] += scale * (double)e;
     }
   }
   __device__ __forceinline__ void direction(CgrShared& sh, T beta) {
@@ -1001,6 +1011,10 @@ __device__ __forceinline__ bool positive(double x) {
   return hi >= 0 && hi <= 0x7ff00000 && (hi | __double2loint(x)) != 0 && !(hi == 0x7ff00000 && __double2loint(x) != 0);
 }
 
+// A search direction is kept over a residual replacement while the true residual is at
+// most 1.1 times the recurrence's (both squared).
+constexpr double KEEP2 = 1.21;
+
 template <class T, class OWN, int NTMAX>
 __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant__ CgrArgs A) {
   extern __shared__ __align__(16) double cgr_dyn[];
@@ -1030,6 +1044,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
     sh.lidx = sh.codes + 2 * A.chunk;
     sh.rsum = sh.lidx + 2 * A.chunk;
     sh.sbody = sh.rsum + A.rcap;
+    sh.held = 0;
   }
   if (A.pl.head[3] != 0) {  // the same for every block
     if (blockIdx.x == 0 && t == 0) {
@@ -1073,6 +1088,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
     load_masses<T>(sh, s);
     const int nwork = (own.work_threads() + 31) >> 5;
     double scale = bnorm;
+    if (t == 0) sh.best = bnorm;
     own.set_r(A, sh, A.rhs, 1.0 / bnorm);
     // the recurrence's r.r below which the true residual is due: a fall by inner_tol
     // or the target, whichever comes first
@@ -1104,6 +1120,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
               sc[0] = al;
               sc[1] = nw * inv;
               sc[2] = z0;
+              sc[3] = rr;
               // 1: the true residual is due; 2: cancellation left no digits of (r.z)', go
               // on from the true residual; 4: no step (p.q or r.z is not positive)
               sh.flag[0] = !(positive(z0) && positive(pq)) ? 4 : (rr <= due ? 1 : (positive(nw) ? 0 : 2));
@@ -1123,7 +1140,12 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
       if (flag != 0 || iters >= A.maxit) {
         // x += scale e; the true FP64 residual replaces r (unit norm) and the search
         // direction is kept with beta in the new units (reliable updates; van der Vorst
-        // and Ye, SIAM J. Sci. Comput. 22 (2000))
+        // and Ye, SIAM J. Sci. Comput. 22 (2000)) -- as long as the recurrence was right:
+        // where it has lost its digits (the late systems of a PDIP run, near the
+        // attainable accuracy) the old direction is not conjugate to the new residual, and
+        // keeping it made FP64 solves diverge (an 8^3 pile's 30th iterate at 1e-12: a
+        // residual of 240 after 20 000 iterations; started afresh 1e-11 after 2200).
+        if (t == 0) sh.keep2 = flag == 1 ? KEEP2 * (double)sc[3] : -1.0;
         own.put_x(A, sh, scale);
         ++N.xc;
         ++N.rc;
@@ -1132,15 +1154,29 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
         ++repl;
         rel = rn / bnorm;
         if (rel <= A.tol) break;
+        const double best = sh.best;
+        const bool better = rn < best;
         if (iters >= A.maxit || repl >= A.max_outer) {
           status = 1;
+          if (!better) {  // the best x that was found, or zero
+            rel = best / bnorm;
+#pragma unroll 1
+            for (long long i = r0 + t; i < r1; i += NT)
+              if (s64.slots == 3 || (i & 3) != 3) A.x[i] = best < bnorm ? A.xbest[i] : 0.0;
+          }
           break;
+        }
+        __syncthreads();
+        if (t == 0) {
+          sh.held = better;
+          if (better) sh.best = rn;
         }
         const double inv = 1.0 / rn;
         own.load(A, sh, s, dinv);
         load_masses<T>(sh, s);
         own.set_r(A, sh, A.r64, inv);
-        beta = flag > 1 ? T(0) : (T)(sh.scal[1] * inv * inv / (double)rz * (rn / scale));
+        const double grew = rn / scale;
+        beta = grew * grew <= sh.keep2 ? (T)(sh.scal[1] * inv * inv / (double)rz * grew) : T(0);
         scale = rn;
         const double goal = A.tol * bnorm * inv;
         due = fmax(drop2, (T)(goal * goal));
@@ -1233,6 +1269,7 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
   A.maxit = maxit;
   A.max_outer = max_outer;
   A.r64 = static_cast<double*>(c->v64[5].ensure((size_t)c->P * sizeof(double)));
+  A.xbest = static_cast<double*>(c->v64[6].ensure((size_t)c->P * sizeof(double)));
   const size_t words = 2 * (size_t)G * CR_HALO * A.rcap + 2 * CR_RED;
   const size_t before = c->cgr_buf.cap;
   u64* buf = static_cast<u64*>(c->cgr_buf.ensure(words * sizeof(u64)));
