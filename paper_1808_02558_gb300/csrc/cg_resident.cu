@@ -1241,7 +1241,7 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
     P.rcap = A.rcap;
     const size_t nb = (size_t)G * A.nbcap, nr = (size_t)G * A.rcap, nc = (size_t)G * 2 * chunk;
     const size_t ints = 4 * (size_t)G + 3 * nb + nr + (size_t)G * G, shorts = 2 * nr + 2 * nc;
-    P.head = static_cast<int*>(c->cgr_plan.ensure(ints * 4 + shorts * 2));
+    P.head = static_cast<int*>(c->cgr.room(c->cgr_plan, ints * 4 + shorts * 2, chunk));
     P.bid = P.head + 4 * (size_t)G;
     P.bmeta = reinterpret_cast<unsigned*>(P.bid + nb);
     P.rmeta = P.bmeta + nb;
@@ -1251,13 +1251,13 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
     P.sbody = P.rsum + nr;
     P.codes = P.sbody + nr;
     P.lidx = P.codes + nc;
-    if (c->cgr_chunk != chunk) {  // no plan yet for this contact set (or one for the other precision)
+    if (c->cgr.chunk != chunk) {  // no plan yet for this contact set (or one for the other precision)
       QP_CUDA(cudaMemsetAsync(P.head, 0, 4 * (size_t)G * sizeof(int), c->stream));
       k_cgr_lists<<<G, 512, 0, c->stream>>>(P, c->M, c->Nc, c->ca.as<int>(), c->cb.as<int>(), c->bptr.as<int>(),
                                             c->inc.as<int>());
       k_cgr_dest<<<G, 512, 0, c->stream>>>(P);
       QP_CUDA(cudaGetLastError());
-      c->cgr_chunk = chunk;
+      c->cgr.chunk = chunk;
     }
   }
   A.rhs = rhs;

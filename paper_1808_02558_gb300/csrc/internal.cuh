@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/qttpdip.h"
+#include "cgr_plan.h"
 
 namespace qp {
 
@@ -107,8 +108,8 @@ struct qp_ctx {
   qp::Buf apart_nb, apart_bodies, apart_cl;
   // exchange slots of the register-resident CG and the next solve's first tag (0: clear the slots first)
   qp::Buf cgr_buf;
-  qp::Buf cgr_plan;    // its plan for the contact set, made for blocks of cgr_chunk contacts (0: none)
-  int cgr_chunk = 0;
+  qp::Buf cgr_plan;    // its plan for the contact set
+  qp::ResidentPlan cgr;
   unsigned cgr_epoch = 0, cgr_last = 0;
   qp::Buf mp_act, mp_w, mp_grad, mp_sum;  // learned warm start: activations, BF16 weights, scratch
   qp::Buf batch64, batch32, batch_table;  // batched solves: per-scene vectors; table (first context)
