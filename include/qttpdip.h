@@ -212,6 +212,14 @@ typedef struct {
 int newton_solve(qp_ctx_t ctx, const qp_state* st, const double* rhs, double* dx,
                  const qp_solve_opts* opts, qp_solve_stats* stats);
 
+/* Which kernel ran the context's last newton_solve or PDIP step's solve: Jacobi-CG runs
+ * with the system held in registers and shared memory (QP_SOLVER_RESIDENT) where it fits,
+ * everything else, and Jacobi-CG of larger or more entangled contact sets, in the
+ * persistent kernel over global memory (QP_SOLVER_GLOBAL).  *resident_launches (may be
+ * NULL): launches of the resident kernel by this context so far, refusals included.      */
+typedef enum { QP_SOLVER_NONE = 0, QP_SOLVER_RESIDENT = 1, QP_SOLVER_GLOBAL = 2 } qp_solver;
+int newton_solver_used(qp_ctx_t ctx, qp_solver* used, int* resident_launches);
+
 /* Batched Newton solves (many independent scenes in one launch): scene i is
  * the current contact set of ctxs[i] with state st[i] (NULL: S = N), solved
  * for rhs[i] -> dx[i] (device, P_i doubles each, not aliased).  The launch is

@@ -21,10 +21,11 @@ QP_NOT_CONVERGED, QP_BREAKDOWN, QP_LINESEARCH_FAIL, QP_TIMEOUT, QP_NOT_READY = -
 QP_F64, QP_F32, QP_BF16 = 0, 1, 2
 QP_JACOBI_PCG, QP_QTT_PCG, QP_QTT_DIRECT = 0, 1, 2
 QP_CG, QP_BICGSTAB = 0, 1
+QP_SOLVER_NONE, QP_SOLVER_RESIDENT, QP_SOLVER_GLOBAL = 0, 1, 2
 QTT_NOALLOC_MAX_VALUES = 1 << 22
 
 SYMBOLS = ["qp_create", "qp_destroy", "qp_status_string", "qp_last_error", "ccp_assemble", "pdip_init",
-           "newton_apply", "newton_rhs", "newton_solve", "newton_solve_batched", "newton_batch_plan", "newton_batch_qtt_tiles", "pdip_step", "pdip_measure", "pdip_solve", "pdip_init_warm",
+           "newton_apply", "newton_rhs", "newton_solve", "newton_solver_used", "newton_solve_batched", "newton_batch_plan", "newton_batch_qtt_tiles", "pdip_step", "pdip_measure", "pdip_solve", "pdip_init_warm",
            "ccp_advance", "qp_selftest_barrier", "mpnn_forward", "mpnn_grad", "mpnn_adam", "mpnn_warm_start", "qtt_from_host",
            "qtt_free", "qtt_get_dims", "qtt_get_ranks", "qtt_copy_cores_to_host", "qtt_apply", "qtt_set_tensor_cores",
            "qtt_round",
@@ -106,6 +107,7 @@ def load(path: str = LIB_PATH):
         "newton_apply": (i, [vp, C.POINTER(State), vp, vp, i]),
         "newton_rhs": (i, [vp, C.POINTER(State), vp]),
         "newton_solve": (i, [vp, C.POINTER(State), vp, vp, C.POINTER(SolveOpts), C.POINTER(SolveStats)]),
+        "newton_solver_used": (i, [vp, C.POINTER(i), C.POINTER(i)]),
         "pdip_step": (i, [vp, C.POINTER(State), C.POINTER(PdipOpts), C.POINTER(PdipStats)]),
         "pdip_measure": (i, [vp, C.POINTER(State), C.POINTER(d), C.POINTER(d)]),
         "pdip_solve": (i, [vp, C.POINTER(State), C.POINTER(PdipOpts), d, d, i, C.POINTER(PdipStats), C.POINTER(i)]),
@@ -346,6 +348,12 @@ class Context:
         self._check(self.lib.newton_solve(self.h, sp, _ptr(rhs), _ptr(dx), C.byref(opts), C.byref(stats)),
                     "newton_solve", allow=allow)
         return stats
+
+    def solver_used(self):
+        """(kernel of the last solve: QP_SOLVER_*, launches of the resident kernel so far)"""
+        used, launches = C.c_int(0), C.c_int(0)
+        self._check(self.lib.newton_solver_used(self.h, C.byref(used), C.byref(launches)), "newton_solver_used")
+        return used.value, launches.value
 
     @staticmethod
     def pdip_opts(solve: SolveOpts, nu=10.0, alpha=0.01, beta=0.5, step_frac=0.99, max_halvings=60, qtt_refresh=0,

@@ -111,6 +111,8 @@ struct qp_ctx {
   qp::Buf cgr_plan;    // its plan for the contact set
   qp::ResidentPlan cgr;
   unsigned cgr_epoch = 0, cgr_last = 0;
+  qp_solver solver_used = QP_SOLVER_NONE;  // kernel of the last solve
+  int cgr_launches = 0;
   qp::Buf mp_act, mp_w, mp_grad, mp_sum;  // learned warm start: activations, BF16 weights, scratch
   qp::Buf batch64, batch32, batch_table;  // batched solves: per-scene vectors; table (first context)
   qp::Buf batch_qw, tune_buf;  // batched QTT work buffers; tile-shape probe data

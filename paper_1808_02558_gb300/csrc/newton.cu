@@ -2526,7 +2526,11 @@ static qp_solve_stats solve_once(qp_ctx* c, const double* rhs, double* dx, const
       QP_CUDA(cudaEventRecord(c->ev1, c->stream));
       const DevCtl h = read_ctl(c);
       if (h.err == 0) c->cgr_epoch = c->cgr_last + (unsigned)h.scal[S_TAGS] + 1u;
-      if (h.err != 0 || h.halvings != CGR_NO_ROOM) return solve_stats(c, h);
+      ++c->cgr_launches;
+      if (h.err != 0 || h.halvings != CGR_NO_ROOM) {
+        c->solver_used = QP_SOLVER_RESIDENT;
+        return solve_stats(c, h);
+      }
     }
   }
   const size_t P = (size_t)c->P;
@@ -2582,6 +2586,7 @@ static qp_solve_stats solve_once(qp_ctx* c, const double* rhs, double* dx, const
   A.ctl = c->ctl.as<DevCtl>();
   A.partial = c->partial.as<double>();
 
+  c->solver_used = QP_SOLVER_GLOBAL;
   reset_ctl(c);
   QP_CUDA(cudaEventRecord(c->ev0, c->stream));
   if (mixed && use_qtt) {
@@ -3029,6 +3034,14 @@ int newton_solve(qp_ctx_t c, const qp_state* st, const double* rhs, double* dx, 
   if (stats) *stats = s;
   if (s.status == QP_TIMEOUT) throw Error{QP_TIMEOUT, "newton_solve: device barrier wait expired"};
   return s.status;
+  API_END(c)
+}
+
+int newton_solver_used(qp_ctx_t c, qp_solver* used, int* resident_launches) {
+  API_BEGIN(c)
+  QP_REQUIRE(used, QP_INVALID_ARG, "newton_solver_used: null result");
+  *used = c->solver_used;
+  if (resident_launches) *resident_launches = c->cgr_launches;
   API_END(c)
 }
 
