@@ -653,7 +653,7 @@ static void assemble(qp_ctx* c, const qp_scene* s, qp_contacts* out) {
   QP_CUDA(cudaStreamSynchronize(st));
   c->have_contacts = true;
   c->apart_G = 0;   // the standalone apply's partition follows the contact set
-  c->cgr = ResidentPlan();  // and so does the resident solver's plan
+  c->cgr.assembled();  // and so does the resident solver's plan
 
   out->M = M;
   out->Nc = Nc;

@@ -51,8 +51,6 @@ namespace {
 typedef unsigned long long u64;
 
 constexpr int CR_MAXG = 256;                   // blocks at most
-constexpr int CR_WR = 9;                        // stride of a contact's wrench in shared memory
-constexpr int CR_WL = 7;                        // stride of a body's intermediate (odd: no bank conflicts)
 constexpr int CR_HALO = 12;                    // tagged words a partial sum (six FP64 values)
 constexpr int CR_RED = 16 * CR_MAXG;           // tagged words of one sum buffer (eight FP64 values a block)
 constexpr int CR_MINT = 256;                   // threads of a block at least
@@ -1193,17 +1191,10 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
   }
 }
 
-// in: with two contacts a thread, p behind the lists
-size_t smem_bytes(const CgrArgs& A, bool in) {
-  return (size_t)A.chunk * (CR_WR * 8 + 8 + (in ? 3 * 4 : 0)) + (size_t)A.nbcap * ((CR_WL + 2) * 8 + 12) +
-         (size_t)A.rcap * (8 + (A.own_rb ? CR_WL * 8 : 0)) + 16;
-}
-
 template <class T, class OWN, int NTMAX>
-bool launch(qp_ctx* c, CgrArgs& A, int G, bool in) {
+bool launch(qp_ctx* c, CgrArgs& A, int G, size_t smem) {
   auto k = k_cg_resident<T, OWN, NTMAX>;
   const int nt = std::max(CR_MINT, (OWN::threads(A.chunk) + 31) / 32 * 32);
-  const size_t smem = smem_bytes(A, in);
   QP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   QP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nt, smem));
@@ -1217,9 +1208,8 @@ bool launch(qp_ctx* c, CgrArgs& A, int G, bool in) {
 
 bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, double inner_tol, int maxit,
                         int max_outer, bool mixed) {
-  constexpr int NT32 = 640, NT1 = 512;
-  const int cap = mixed ? 2 * NT32 : NT1;  // contacts a block
-  if (c->Nc < 1 || c->num_sms > CR_MAXG) return false;
+  const int cap = mixed ? CR_CHUNK2 : CR_CHUNK1;  // contacts a block
+  if (c->Nc < 1 || c->num_sms > CR_MAXG || c->cgr.tried[mixed] == ResidentPlan::NONE) return false;
   // no fewer contacts a block than fill its four schedulers once (a warp each; FP64
   // with four lanes a contact): more blocks would only make the sums longer
   const int chunk = std::max(ceil_div(c->Nc, c->num_sms), mixed ? 128 : 32);
@@ -1229,11 +1219,14 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
   A.s64 = view64(c, true);
   A.s32 = view32(c, true);
   A.chunk = chunk;
-  // room for lists: the 40^3 pile (1262 contacts a block) needs 654 bodies and 549 runs
-  A.own_rb = chunk <= NT1 ? 1 : 0;
-  A.nbcap = std::min(2 * chunk, A.own_rb ? 960 : 800);
-  // (rcap even: 32-bit data follows two 16-bit lists of that length in shared memory)
-  A.rcap = A.own_rb ? std::min(std::max(256, 2 * chunk), 1024) : (chunk * CR_WR / CR_WL) & ~1;
+  int optin = 0;
+  QP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+  const ResidentShape shape = resident_shape(chunk, (size_t)std::max(0, optin - (int)sizeof(CgrShared) - 256),
+                                             c->cgr.tried[mixed] == ResidentPlan::ALL);
+  c->cgr_full = shape.full;
+  A.own_rb = shape.own_rb;
+  A.nbcap = shape.nbcap;
+  A.rcap = shape.rcap;
   {
     CgrPlan& P = A.pl;
     P.chunk = chunk;
@@ -1287,10 +1280,10 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
   bool ok;
   // FP64: a row a lane while that keeps every FP64 unit at one warp or two (64 contacts
   // an SM); above, a contact a thread fills the units as well with fewer instructions
-  if (!mixed && chunk <= 64) ok = launch<double, Rows<double>, 256>(c, A, G, false);
-  else if (!mixed) ok = launch<double, Own<double, 1>, NT1>(c, A, G, false);
-  else if (chunk <= NT1) ok = launch<float, Own<float, 1>, NT1>(c, A, G, false);
-  else ok = launch<float, Own<float, 2>, NT32>(c, A, G, true);
+  if (!mixed && chunk <= 64) ok = launch<double, Rows<double>, 256>(c, A, G, shape.smem());
+  else if (!mixed) ok = launch<double, Own<double, 1>, CR_CHUNK1>(c, A, G, shape.smem());
+  else if (chunk <= CR_CHUNK1) ok = launch<float, Own<float, 1>, CR_CHUNK1>(c, A, G, shape.smem());
+  else ok = launch<float, Own<float, 2>, CR_CHUNK2 / 2>(c, A, G, shape.smem());
   if (!ok) c->cgr_epoch = A.epoch;
   return ok;
 }

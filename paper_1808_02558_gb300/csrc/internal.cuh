@@ -110,6 +110,7 @@ struct qp_ctx {
   qp::Buf cgr_buf;
   qp::Buf cgr_plan;    // its plan for the contact set
   qp::ResidentPlan cgr;
+  bool cgr_full = false;  // the last plan had all the room
   unsigned cgr_epoch = 0, cgr_last = 0;
   qp_solver solver_used = QP_SOLVER_NONE;  // kernel of the last solve
   int cgr_launches = 0;

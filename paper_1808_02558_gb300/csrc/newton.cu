@@ -2517,21 +2517,23 @@ static qp_solve_stats solve_once(qp_ctx* c, const double* rhs, double* dx, const
                                                 c->P);
   QP_CUDA(cudaGetLastError());
   // Jacobi-PCG: the register-resident kernel where the system fits the SMs (up to
-  // 1280 contacts an SM mixed, 512 in FP64), the classic kernel otherwise
-  if (!use_qtt && o->krylov != QP_BICGSTAB) {
+  // 1280 contacts an SM mixed, 512 in FP64, and its plan finds room), the global kernel
+  // otherwise
+  while (!use_qtt && o->krylov != QP_BICGSTAB) {
     reset_ctl(c);
     QP_CUDA(cudaEventRecord(c->ev0, c->stream));
-    if (launch_cg_resident(c, rhs, dx, o->tol, o->inner_tol > 0 ? o->inner_tol : (mixed ? 1e-4 : o->tol), o->maxit,
-                           o->max_outer > 0 ? o->max_outer : (mixed ? 50 : 5), mixed)) {
-      QP_CUDA(cudaEventRecord(c->ev1, c->stream));
-      const DevCtl h = read_ctl(c);
-      if (h.err == 0) c->cgr_epoch = c->cgr_last + (unsigned)h.scal[S_TAGS] + 1u;
-      ++c->cgr_launches;
-      if (h.err != 0 || h.halvings != CGR_NO_ROOM) {
-        c->solver_used = QP_SOLVER_RESIDENT;
-        return solve_stats(c, h);
-      }
+    if (!launch_cg_resident(c, rhs, dx, o->tol, o->inner_tol > 0 ? o->inner_tol : (mixed ? 1e-4 : o->tol), o->maxit,
+                            o->max_outer > 0 ? o->max_outer : (mixed ? 50 : 5), mixed))
+      break;
+    QP_CUDA(cudaEventRecord(c->ev1, c->stream));
+    const DevCtl h = read_ctl(c);
+    if (h.err == 0) c->cgr_epoch = c->cgr_last + (unsigned)h.scal[S_TAGS] + 1u;
+    ++c->cgr_launches;
+    if (h.err != 0 || h.halvings != CGR_NO_ROOM) {
+      c->solver_used = QP_SOLVER_RESIDENT;
+      return solve_stats(c, h);
     }
+    c->cgr.refused(mixed, c->cgr_full);
   }
   const size_t P = (size_t)c->P;
   PcgArgs A;

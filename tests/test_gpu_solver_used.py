@@ -8,7 +8,7 @@ import torch
 from gpu_common import dev, to_np
 from oracle import contacts as oc, qp
 from paper_1808_02558_gb300 import binding, workload
-from synth import Scene, lattice_scene
+from synth import Scene, box_scene, lattice_scene
 
 pytestmark = pytest.mark.gpu
 
@@ -91,3 +91,16 @@ def test_mixed_beyond_the_room():
 def test_refused_by_the_plan(mixed):
     (used, launches), _ = solve(studded_ball(), mixed, 1e-10, again=2)
     assert used == binding.QP_SOLVER_GLOBAL and launches >= 1
+
+
+@pytest.mark.parametrize("mixed", [0, 1])
+def test_a_refusal_is_remembered(mixed):
+    scene = studded_ball()
+    assert solve(scene, mixed, 1e-8, again=1)[0] == solve(scene, mixed, 1e-8, again=4)[0]
+
+
+def test_sparse_contact_sets_are_resident():
+    """A walled box of 55^3 falling spheres has about one body a contact, more than the usual
+    room of a block holds: the second shape takes it, and the next solve goes there at once."""
+    used, Nc = solve(box_scene(5, n=55, layers=55), 1, 1e-10, again=3)
+    assert used == (binding.QP_SOLVER_RESIDENT, 4)

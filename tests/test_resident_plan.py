@@ -67,3 +67,41 @@ def test_plan_is_disowned_when_its_buffer_cannot_grow(tmp_path):
   std::free(b.p);
 """)
     assert out == ["128", "0", "0", "0"]
+
+
+def test_room_of_a_block(tmp_path):
+    """Lists fit the shared memory at every size, hold every contact set up to 512 contacts a
+    block, and with all the room the walled boxes that the plan's counts were taken from."""
+    out = run(tmp_path, r"""
+  const size_t room = 232448 - 4400 - 256;  // a block's most on sm_103a, less the static part
+  for (int all = 0; all < 2; ++all)
+    for (int chunk = 1; chunk <= qp::CR_CHUNK2; ++chunk) {
+      const qp::ResidentShape s = qp::resident_shape(chunk, room, all);
+      if (s.smem() > room || s.rcap % 2 || s.nbcap < 1) std::printf("bad-%d-%d ", all, chunk);
+      if (chunk <= qp::CR_CHUNK1 && (s.nbcap != 2 * chunk || s.rcap < 2 * chunk || !s.full)) std::printf("short-%d ", chunk);
+      if (chunk > qp::CR_CHUNK1 && !s.own_rb && s.rcap * qp::CR_WL > chunk * qp::CR_WR) std::printf("alias-%d ", chunk);
+      if (all && !s.full) std::printf("full-%d ", chunk);
+    }
+  // contacts and bodies a block of walled boxes of 52, 55, 58 and 60 spheres a side
+  const int need[4][2] = {{805, 810}, {944, 935}, {1101, 1074}, {1214, 1179}};
+  for (auto& n : need) std::printf("%d", qp::resident_shape(n[0], room, true).nbcap >= n[1]);
+  // no room at all
+  std::printf(" %d\n", qp::resident_shape(1280, 1000, true).nbcap);
+""")
+    assert out == ["1111", "0"]
+
+
+def test_refusals_are_remembered_for_the_contact_set(tmp_path):
+    out = run(tmp_path, r"""
+  using P = qp::ResidentPlan;
+  P c;
+  c.chunk = 900;
+  c.refused(true, false);   // the usual room was too small: all of it next, with another plan
+  std::printf("%d%d%d ", c.chunk, c.tried[0] == P::USUAL, c.tried[1] == P::ALL);
+  c.chunk = 900;
+  c.refused(true, true);    // and so was all of it
+  std::printf("%d%d%d ", c.chunk, c.tried[0] == P::USUAL, c.tried[1] == P::NONE);
+  c.assembled();
+  std::printf("%d%d\n", c.tried[0] == P::USUAL, c.tried[1] == P::ALL);
+""")
+    assert out == ["011", "011", "11"]
