@@ -87,7 +87,7 @@ struct CgrArgs {
   int maxit, max_outer;
   unsigned epoch;        // first tag of this solve
   double* r64;           // [P] FP64 residual
-  double* xbest;         // [P] the replaced x of the smallest true residual, while x is not it
+  double* xbest;         // [P] the x of the smallest true residual so far
   u64* halo;             // [2][G][CR_HALO / 2][rcap][2] inboxes, pairs of words by place
   u64* red;              // [2][CR_RED]
   DevCtl* ctl;
@@ -140,9 +140,12 @@ struct CgrShared {
   double poll[32][8];           // per warp: sums over its share of the blocks' messages
   double scal[8];                // what the sum's last step hands to the block
   int flag[2];
+  // what only a replacement uses (in registers it would be spilled around the iterations)
+  double bnorm, scale;           // ||rhs||, and r's unit
+  double rz;                     // r.z of the iteration before
+  double rel;                    // true relative residual (thread 0)
   double best;                   // smallest true residual norm so far
   double keep2;                  // squared growth of the residual up to which the direction is kept
-  int held;                      // x is the (nonzero) solution that has it
   // the block's lists (CgrPlan's, in shared memory)
   int c0, c1, chunk, nbcap, rcap, nbord, nint, nrem;
   double* wr;             // [chunk][CR_WR] wrenches of the block's contacts (viewed as T)
@@ -784,25 +787,21 @@ struct Own {
         for (int u = 0; u < 3; ++u) r[k][u] = (T)(v[row + u] * inv);
       }
   }
-  // x += scale e, the best x aside (and p, where it is not kept in registers over a residual)
+  // x += scale e (and p aside, where it is not kept in registers over a residual)
   __device__ __forceinline__ void put_x(const CgrArgs& A, CgrShared& sh, double scale) {
-    const bool held = sh.held;
 #pragma unroll
     for (int k = 0; k < KC; ++k)
       if (on(k)) {
         const int lc = t + k * NT;
-        const long long row = (long long)A.s64.slots * (sh.c0 + lc);
-        double* x = A.x + row;
-        const double old[3] = {x[0], x[1], x[2]};  // all loads before a store
+        double* x = A.x + (long long)A.s64.slots * (sh.c0 + lc);
 #pragma unroll
         for (int u = 0; u < 3; ++u) {
           if constexpr (SM) {
-            x[u] = old[u] + scale * (double)es[3 * lc + u];
+            x[u] += scale * (double)es[3 * lc + u];
             ps[3 * lc + u] = pr[k][u];
           } else {
-            x[u] = old[u] + scale * (double)er[k][u];
+            x[u] += scale * (double)er[k][u];
           }
-          if (held) A.xbest[row + u] = old[u];
         }
       }
   }
@@ -942,9 +941,7 @@ struct Rows {
   }
   __device__ __forceinline__ void put_x(const CgrArgs& A, CgrShared& sh, double scale) {
     if (act) {
-      const long long row = (long long)A.s64.slots * (sh.c0 + lc) + u;
-      if (sh.held) A.xbest[row] = A.x[row];
-      A.x[row] += scale * (double)e;
+      A.x[(long long)A.s64.slots * (sh.c0 + lc) + u] += scale * (double)e;
     }
   }
   __device__ __forceinline__ void direction(CgrShared& sh, T beta) {
@@ -1009,6 +1006,19 @@ __device__ __forceinline__ bool positive(double x) {
   return hi >= 0 && hi <= 0x7ff00000 && (hi | __double2loint(x)) != 0 && !(hi == 0x7ff00000 && __double2loint(x) != 0);
 }
 
+// to = from (0 without one) in the block's rows but for the identity rows of four slots.
+// Out of line, as residual() is.
+__device__ __noinline__ void copy_rows(const CgrArgs& A, const CgrShared& sh, const double* __restrict__ from,
+                                       double* __restrict__ to) {
+  const int slots = A.s64.slots;
+  const long long r1 = (long long)slots * sh.c1;
+#pragma unroll 4
+  for (long long i = (long long)slots * sh.c0 + threadIdx.x; i < r1; i += blockDim.x) {
+    const double v = from ? from[i] : 0.0;
+    if (slots == 3 || (i & 3) != 3) to[i] = v;
+  }
+}
+
 // A search direction is kept over a residual replacement while the true residual is at
 // most 1.1 times the recurrence's (both squared).
 constexpr double KEEP2 = 1.21;
@@ -1042,7 +1052,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
     sh.lidx = sh.codes + 2 * A.chunk;
     sh.rsum = sh.lidx + 2 * A.chunk;
     sh.sbody = sh.rsum + A.rcap;
-    sh.held = 0;
   }
   if (A.pl.head[3] != 0) {  // the same for every block
     if (blockIdx.x == 0 && t == 0) {
@@ -1078,15 +1087,17 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
   if (!all_sum_cold(A.red + (size_t)(N.rc & 1) * CR_RED, A.ctl, A.epoch + N.rc, sh, b0, 0.0)) return;
   const double bnorm = sqrt(sh.scal[0]);
   int iters = 0, repl = 0, status = 0;
-  double rel = 0.0;
+  if (t == 0) {
+    sh.bnorm = bnorm;
+    sh.rel = 0.0;
+  }
   if (bnorm != 0.0) {
     OWN own;
     own.load(A, sh, s, dinv);
     own.zero_p();
     load_masses<T>(sh, s);
     const int nwork = (own.work_threads() + 31) >> 5;
-    double scale = bnorm;
-    if (t == 0) sh.best = bnorm;
+    if (t == 0) sh.scale = sh.best = bnorm;
     own.set_r(A, sh, A.rhs, 1.0 / bnorm);
     // the recurrence's r.r below which the true residual is due: a fall by inner_tol
     // or the target, whichever comes first
@@ -1126,7 +1137,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
           }))
         return;
       const int flag = sh.flag[0];
-      const T rz = sc[2];
       beta = sc[1];
       if (flag != 4) {
         own.step(sc[0]);
@@ -1143,40 +1153,39 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
         // attainable accuracy) the old direction is not conjugate to the new residual, and
         // keeping it made FP64 solves diverge (an 8^3 pile's 30th iterate at 1e-12: a
         // residual of 240 after 20 000 iterations; started afresh 1e-11 after 2200).
-        if (t == 0) sh.keep2 = flag == 1 ? KEEP2 * (double)sc[3] : -1.0;
-        own.put_x(A, sh, scale);
+        if (t == 0) {
+          sh.rz = (double)sc[2];
+          sh.keep2 = flag == 1 ? KEEP2 * (double)sc[3] : -1.0;
+        }
+        own.put_x(A, sh, sh.scale);
         ++N.xc;
         ++N.rc;
         if (!residual(A, N.xc, N.rc, sh)) return;
         const double rn = sqrt(sh.scal[0]);
         ++repl;
-        rel = rn / bnorm;
-        if (rel <= A.tol) break;
-        const double best = sh.best;
-        const bool better = rn < best;
+        if (t == 0) sh.rel = rn / sh.bnorm;
+        if (rn / sh.bnorm <= A.tol) break;
         if (iters >= A.maxit || repl >= A.max_outer) {
           status = 1;
-          if (!better) {  // the best x that was found, or zero
-            rel = best / bnorm;
-#pragma unroll 1
-            for (long long i = r0 + t; i < r1; i += NT)
-              if (s64.slots == 3 || (i & 3) != 3) A.x[i] = best < bnorm ? A.xbest[i] : 0.0;
+          if (!(rn < sh.best)) {  // the best x that was found, or zero
+            if (t == 0) sh.rel = sh.best / sh.bnorm;
+            copy_rows(A, sh, sh.best < sh.bnorm ? A.xbest : nullptr, A.x);
           }
           break;
         }
-        __syncthreads();
-        if (t == 0) {
-          sh.held = better;
-          if (better) sh.best = rn;
-        }
+        if (rn < sh.best) copy_rows(A, sh, A.x, A.xbest);  // (the same in every thread)
         const double inv = 1.0 / rn;
         own.load(A, sh, s, dinv);
         load_masses<T>(sh, s);
         own.set_r(A, sh, A.r64, inv);
-        const double grew = rn / scale;
-        beta = grew * grew <= sh.keep2 ? (T)(sh.scal[1] * inv * inv / (double)rz * grew) : T(0);
-        scale = rn;
-        const double goal = A.tol * bnorm * inv;
+        const double grew = rn / sh.scale;
+        beta = grew * grew <= sh.keep2 ? (T)(sh.scal[1] * inv * inv / sh.rz * grew) : T(0);
+        __syncthreads();
+        if (t == 0) {
+          sh.scale = rn;
+          if (rn < sh.best) sh.best = rn;
+        }
+        const double goal = A.tol * sh.bnorm * inv;
         due = fmax(drop2, (T)(goal * goal));
       }
     }
@@ -1184,8 +1193,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
   if (blockIdx.x == 0 && t == 0) {
     A.ctl->iters = iters;
     A.ctl->outer = repl;
-    A.ctl->scal[S_RELRES] = rel;
-    A.ctl->scal[S_BNORM] = bnorm;
+    A.ctl->scal[S_RELRES] = sh.rel;
+    A.ctl->scal[S_BNORM] = sh.bnorm;
     A.ctl->scal[S_TAGS] = (double)(N.rc > N.xc ? N.rc : N.xc);
     A.ctl->halvings = status;
   }
