@@ -628,7 +628,8 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// (hi, lo) += v with the rounding error kept (Knuth's TwoSum)
+// (hi, lo) += v with the rounding error kept (Knuth's TwoSum); lo is NaN from the first
+// hi on that is not finite
 __device__ __forceinline__ void fold(float& hi, float& lo, float v) {
   const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
   lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
@@ -639,8 +640,10 @@ __device__ __forceinline__ void fold(float& hi, float& lo, float v) {
 // a block takes 32 outputs, its 32 warps a share of the partials each, added in
 // warp order in FP64.  A warp's share is summed in FP32 with the rounding errors kept:
 // converting and adding the 7 M partials of a layer on the FP64 pipe takes 22 us by
-// itself.  12 us on average; a thread an output, its partials one after the other,
-// took 127.
+// itself, and a third term (70 bits) changes no gradient but takes 14 us over the five
+// sums.  A share with an infinite partial, or whose running sum leaves FP32's range, is
+// summed again in FP64.  12 us on average; a thread an output, its partials one after the
+// other, took 127.
 __global__ void __launch_bounds__(1024)
     k_wgrad_sum(int nparts, int J, int K, const float* __restrict__ part, float* __restrict__ gW,
                 float* __restrict__ gb) {
@@ -648,12 +651,18 @@ __global__ void __launch_bounds__(1024)
   const int n = J * (K + 1), lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int o = blockIdx.x * 32 + lane;
   const int g0 = (int)((long long)nparts * w / 32), g1 = (int)((long long)nparts * (w + 1) / 32);
-  float hi = 0.f, lo = 0.f;
+  double share = 0.0;
   if (o < n) {
+    float hi = 0.f, lo = 0.f;
 #pragma unroll 8
     for (int g = g0; g < g1; ++g) fold(hi, lo, __ldg(part + (size_t)g * n + o));
+    if (lo == lo) {
+      share = (double)hi + (double)lo;
+    } else {
+      for (int g = g0; g < g1; ++g) share += (double)__ldg(part + (size_t)g * n + o);
+    }
   }
-  sm[w][lane] = (double)hi + (double)lo;
+  sm[w][lane] = share;
   __syncthreads();
   if (w == 0 && o < n) {
     double s = 0.0;
