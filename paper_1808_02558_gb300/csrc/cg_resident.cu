@@ -1201,10 +1201,13 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
 }
 
 template <class T, class OWN, int NTMAX>
-bool launch(qp_ctx* c, CgrArgs& A, int G, size_t smem) {
+bool launch(qp_ctx* c, CgrArgs& A, int G, size_t smem, size_t room) {
   auto k = k_cg_resident<T, OWN, NTMAX>;
   const int nt = std::max(CR_MINT, (OWN::threads(A.chunk) + 31) / 32 * 32);
-  QP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (smem > room) return false;
+  // the limit belongs to the function, not to the launch: always all the room, or another
+  // thread's smaller system could lower it before this launch
+  QP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
   int per_sm = 0;
   QP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nt, smem));
   if (per_sm < 1) return false;
@@ -1230,8 +1233,8 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
   A.chunk = chunk;
   int optin = 0;
   QP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-  const ResidentShape shape = resident_shape(chunk, (size_t)std::max(0, optin - (int)sizeof(CgrShared) - 256),
-                                             c->cgr.tried[mixed] == ResidentPlan::ALL);
+  const size_t room = (size_t)std::max(0, optin - (int)sizeof(CgrShared) - 256);
+  const ResidentShape shape = resident_shape(chunk, room, c->cgr.tried[mixed] == ResidentPlan::ALL);
   c->cgr_full = shape.full;
   A.own_rb = shape.own_rb;
   A.nbcap = shape.nbcap;
@@ -1289,10 +1292,10 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
   bool ok;
   // FP64: a row a lane while that keeps every FP64 unit at one warp or two (64 contacts
   // an SM); above, a contact a thread fills the units as well with fewer instructions
-  if (!mixed && chunk <= 64) ok = launch<double, Rows<double>, 256>(c, A, G, shape.smem());
-  else if (!mixed) ok = launch<double, Own<double, 1>, CR_CHUNK1>(c, A, G, shape.smem());
-  else if (chunk <= CR_CHUNK1) ok = launch<float, Own<float, 1>, CR_CHUNK1>(c, A, G, shape.smem());
-  else ok = launch<float, Own<float, 2>, CR_CHUNK2 / 2>(c, A, G, shape.smem());
+  if (!mixed && chunk <= 64) ok = launch<double, Rows<double>, 256>(c, A, G, shape.smem(), room);
+  else if (!mixed) ok = launch<double, Own<double, 1>, CR_CHUNK1>(c, A, G, shape.smem(), room);
+  else if (chunk <= CR_CHUNK1) ok = launch<float, Own<float, 1>, CR_CHUNK1>(c, A, G, shape.smem(), room);
+  else ok = launch<float, Own<float, 2>, CR_CHUNK2 / 2>(c, A, G, shape.smem(), room);
   if (!ok) c->cgr_epoch = A.epoch;
   return ok;
 }
