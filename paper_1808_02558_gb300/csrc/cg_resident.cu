@@ -134,6 +134,10 @@ __device__ __forceinline__ T wsum8(const T (&v)[8]) {
   return c + __shfl_xor_sync(0xffffffffu, c, 1);
 }
 
+// What a residual replacement finds: the tolerance is met; a cap is, at the smallest
+// residual so far or after a smaller one; neither, at the smallest so far or not.
+enum { R_DONE, R_CAP, R_CAP_BACK, R_KEEP, R_GO };
+
 // Shared-memory state of a block beside the dynamic arrays.
 struct CgrShared {
   double part[32][8];            // per warp: sums over its threads
@@ -143,8 +147,11 @@ struct CgrShared {
   // what only a replacement uses (in registers it would be spilled around the iterations)
   double bnorm, scale;           // ||rhs||, and r's unit
   double rz;                     // r.z of the iteration before
-  double rel;                    // true relative residual (thread 0)
+  double rel;                    // true relative residual
   double best;                   // smallest true residual norm so far
+  int kept;                      // its x is in A.xbest (else it is 0)
+  double inv, beta, due;         // r's new scaling, the next beta, the next due r.r
+  int next;                      // R_*: what a replacement found
   double keep2;                  // squared growth of the residual up to which the direction is kept
   // the block's lists (CgrPlan's, in shared memory)
   int c0, c1, chunk, nbcap, rcap, nbord, nint, nrem;
@@ -1071,40 +1078,43 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
     if constexpr (sizeof(T) == 4) return A.dinv32;
     else return A.dinv64;
   }();
-  double b0 = 0.0;
+  double b0 = 0.0, b1 = 0.0;  // the right-hand side's squares: all rows, and those left to solve
   const long long r0 = (long long)s64.slots * sh.c0, r1 = (long long)s64.slots * sh.c1;
 #pragma unroll 1
   for (long long i = r0 + t; i < r1; i += NT) {
     const double bi = A.rhs[i];
-    b0 += bi * bi;
     // with four slots the last row is an identity row: solved by its right-hand side
-    A.x[i] = (s64.slots == 4 && (i & 3) == 3) ? bi : 0.0;
+    const bool solved = s64.slots == 4 && (i & 3) == 3;
+    b0 += bi * bi;
+    if (!solved) b1 += bi * bi;
+    A.x[i] = solved ? bi : 0.0;
   }
 #pragma unroll 1
   for (long long i = (long long)s64.slots * s64.Nc + blockIdx.x * (long long)NT + t; i < s64.P; i += (long long)G * NT)
     A.x[i] = 0.0;
   ++N.rc;
-  if (!all_sum_cold(A.red + (size_t)(N.rc & 1) * CR_RED, A.ctl, A.epoch + N.rc, sh, b0, 0.0)) return;
-  const double bnorm = sqrt(sh.scal[0]);
-  int iters = 0, repl = 0, status = 0;
+  if (!all_sum_cold(A.red + (size_t)(N.rc & 1) * CR_RED, A.ctl, A.epoch + N.rc, sh, b0, b1)) return;
   if (t == 0) {
-    sh.bnorm = bnorm;
-    sh.rel = 0.0;
+    sh.bnorm = sh.scale = sqrt(sh.scal[0]);
+    sh.best = sqrt(sh.scal[1]);
+    sh.rel = sh.bnorm == 0.0 ? 0.0 : sh.best / sh.bnorm;
+    sh.kept = 0;
   }
-  if (bnorm != 0.0) {
+  __syncthreads();
+  int iters = 0, repl = 0, status = 0;
+  if (!(sh.rel <= A.tol)) {
     OWN own;
     own.load(A, sh, s, dinv);
     own.zero_p();
     load_masses<T>(sh, s);
     const int nwork = (own.work_threads() + 31) >> 5;
-    if (t == 0) sh.scale = sh.best = bnorm;
-    own.set_r(A, sh, A.rhs, 1.0 / bnorm);
+    own.set_r(A, sh, A.rhs, 1.0 / sh.bnorm);
     // the recurrence's r.r below which the true residual is due: a fall by inner_tol
     // or the target, whichever comes first
     const T drop2 = (T)(A.inner_tol * A.inner_tol);
     T due = fmax(drop2, (T)(A.tol * A.tol));
     T beta = T(0);
-    T* sc = reinterpret_cast<T*>(sh.scal);  // alpha, beta, r.z
+    T* sc = reinterpret_cast<T*>(sh.scal);  // alpha, beta, r.z, the new r.r
     for (;;) {
       if (iters >= A.maxit) {
         status = 1;
@@ -1161,32 +1171,36 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
         ++N.xc;
         ++N.rc;
         if (!residual(A, N.xc, N.rc, sh)) return;
-        const double rn = sqrt(sh.scal[0]);
         ++repl;
-        if (t == 0) sh.rel = rn / sh.bnorm;
-        if (rn / sh.bnorm <= A.tol) break;
-        if (iters >= A.maxit || repl >= A.max_outer) {
+        // by one thread: a dozen warps' square roots and divisions would take their turn
+        // in the SM's narrow FP64 pipe
+        if (t == 0) {
+          const double rn = sqrt(sh.scal[0]), rel = rn / sh.bnorm, inv = 1.0 / rn, grew = rn / sh.scale;
+          const double goal = A.tol * sh.bnorm * inv;
+          const bool better = rn < sh.best, last = iters >= A.maxit || repl >= A.max_outer;
+          sh.next = rel <= A.tol ? R_DONE : (last ? (better ? R_CAP : R_CAP_BACK) : (better ? R_KEEP : R_GO));
+          sh.rel = last && !better ? sh.best / sh.bnorm : rel;
+          sh.inv = inv;
+          sh.beta = grew * grew <= sh.keep2 ? sh.scal[1] * inv * inv / sh.rz * grew : 0.0;
+          sh.due = goal * goal;
+          sh.scale = rn;
+          if (better) sh.best = rn;
+          if (sh.next == R_KEEP) sh.kept = 1;
+        }
+        __syncthreads();
+        const int next = sh.next;
+        if (next == R_DONE) break;
+        if (next == R_CAP || next == R_CAP_BACK) {
           status = 1;
-          if (!(rn < sh.best)) {  // the best x that was found, or zero
-            if (t == 0) sh.rel = sh.best / sh.bnorm;
-            copy_rows(A, sh, sh.best < sh.bnorm ? A.xbest : nullptr, A.x);
-          }
+          if (next == R_CAP_BACK) copy_rows(A, sh, sh.kept ? A.xbest : nullptr, A.x);
           break;
         }
-        if (rn < sh.best) copy_rows(A, sh, A.x, A.xbest);  // (the same in every thread)
-        const double inv = 1.0 / rn;
+        if (next == R_KEEP) copy_rows(A, sh, A.x, A.xbest);
         own.load(A, sh, s, dinv);
         load_masses<T>(sh, s);
-        own.set_r(A, sh, A.r64, inv);
-        const double grew = rn / sh.scale;
-        beta = grew * grew <= sh.keep2 ? (T)(sh.scal[1] * inv * inv / sh.rz * grew) : T(0);
-        __syncthreads();
-        if (t == 0) {
-          sh.scale = rn;
-          if (rn < sh.best) sh.best = rn;
-        }
-        const double goal = A.tol * sh.bnorm * inv;
-        due = fmax(drop2, (T)(goal * goal));
+        own.set_r(A, sh, A.r64, sh.inv);
+        beta = (T)sh.beta;
+        due = fmax(drop2, (T)sh.due);
       }
     }
   }
