@@ -349,6 +349,18 @@ int pdip_solve(qp_ctx_t ctx, qp_state* st, const qp_pdip_opts* opts, double gap_
  * the kernels' own budget (4e9 ticks) and absent_block < the SM count.       */
 int qp_selftest_barrier(qp_ctx_t ctx, long long budget, int absent_block, int* device_status);
 
+/* The same for the resident solver's waits, which are bounded polls of data that other
+ * blocks send: one iteration on N dx = rhs (double[P] each, not aliased) for the current
+ * contact set, which has to fit the resident solver, in FP64 or mixed precision, in which
+ * block absent_block leaves before the first sum over the blocks (at = 0) or before the
+ * first exchange between neighbours (at = 1).  The others' waits expire after `polls`
+ * polls; *device_status is QP_TIMEOUT then, and QP_OK otherwise (absent_block < 0: all
+ * take part).  The launch always ends, and the context's next solve is as any other.
+ * QP_INVALID_ARG unless 0 < polls <= the solver's own (2^22), absent_block < the SM
+ * count, at is 0 or 1 and the contact set is resident.                       */
+int qp_selftest_resident(qp_ctx_t ctx, const double* rhs, double* dx, int mixed, int polls, int absent_block, int at,
+                         int* device_status);
+
 /* ---- Learned warm start (an extension; the paper has no counterpart) ---- */
 
 /* A message-passing network over the contact graph predicts the impulses the

@@ -26,7 +26,7 @@ QTT_NOALLOC_MAX_VALUES = 1 << 22
 
 SYMBOLS = ["qp_create", "qp_destroy", "qp_status_string", "qp_last_error", "ccp_assemble", "pdip_init",
            "newton_apply", "newton_rhs", "newton_solve", "newton_solver_used", "newton_solve_batched", "newton_batch_plan", "newton_batch_qtt_tiles", "pdip_step", "pdip_measure", "pdip_solve", "pdip_init_warm",
-           "ccp_advance", "qp_selftest_barrier", "mpnn_forward", "mpnn_grad", "mpnn_adam", "mpnn_warm_start", "qtt_from_host",
+           "ccp_advance", "qp_selftest_barrier", "qp_selftest_resident", "mpnn_forward", "mpnn_grad", "mpnn_adam", "mpnn_warm_start", "qtt_from_host",
            "qtt_free", "qtt_get_dims", "qtt_get_ranks", "qtt_copy_cores_to_host", "qtt_apply", "qtt_set_tensor_cores",
            "qtt_round",
            "qtt_compress", "qtt_inverse", "qtt_apply_f32_noalloc"]
@@ -118,6 +118,7 @@ def load(path: str = LIB_PATH):
         "newton_batch_qtt_tiles": (i, [vp, i, C.POINTER(i)]),
         "ccp_advance": (i, [vp, C.POINTER(Scene), C.POINTER(State), vp, vp, vp]),
         "qp_selftest_barrier": (i, [vp, ll, i, C.POINTER(i)]),
+        "qp_selftest_resident": (i, [vp, vp, vp, i, i, i, i, C.POINTER(i)]),
         "mpnn_forward": (i, [vp, vp, C.POINTER(C.c_float), vp]),
         "mpnn_grad": (i, [vp, vp, C.POINTER(C.c_float), vp, vp, C.POINTER(d)]),
         "mpnn_adam": (i, [vp, vp, vp, vp, vp, i, d, d, d, d]),
@@ -288,6 +289,13 @@ class Context:
         status = C.c_int(0)
         self._check(self.lib.qp_selftest_barrier(self.h, int(budget), int(absent_block), C.byref(status)),
                     "qp_selftest_barrier")
+        return status.value
+
+    def selftest_resident(self, rhs, dx, mixed: int, polls: int, absent_block: int, at: int = 0) -> int:
+        """Device status of a resident iteration that one block leaves."""
+        status = C.c_int(0)
+        self._check(self.lib.qp_selftest_resident(self.h, _ptr(rhs), _ptr(dx), int(mixed), int(polls),
+                                                  int(absent_block), int(at), C.byref(status)), "qp_selftest_resident")
         return status.value
 
     # ------------------------------------------------------------- learned warm start

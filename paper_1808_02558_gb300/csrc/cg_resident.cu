@@ -86,6 +86,9 @@ struct CgrArgs {
   double tol, inner_tol;
   int maxit, max_outer;
   unsigned epoch;        // first tag of this solve
+  unsigned polls;        // unsuccessful polls after which a wait expires
+  int absent;            // self-test: block that leaves (-1: none) ...
+  int absent_at;         // ... before the first sum (0) or the first exchange (1)
   double* r64;           // [P] FP64 residual
   double* xbest;         // [P] the x of the smallest true residual so far
   u64* halo;             // [2][G][CR_HALO / 2][rcap][2] inboxes, pairs of words by place
@@ -106,10 +109,9 @@ __device__ __forceinline__ u64 word(unsigned bits, unsigned tag) { return ((u64)
 __device__ __forceinline__ unsigned tag_of(u64 w) { return (unsigned)(w >> 32); }
 
 // One more unsuccessful poll (each takes an L2 round trip, at least 400 cycles); true:
-// leave, because the wait expired (about a second) or another block failed.
-constexpr unsigned CR_SPINS = 4u << 20;
-__device__ __forceinline__ bool give_up(DevCtl* ctl, unsigned& spins) {
-  return ++spins > CR_SPINS || ((spins & 1023u) == 0 && *(volatile int*)&ctl->err != 0);
+// leave, because the wait expired or another block failed.
+__device__ __forceinline__ bool give_up(DevCtl* ctl, unsigned& spins, unsigned polls) {
+  return ++spins > polls || ((spins & 1023u) == 0 && *(volatile int*)&ctl->err != 0);
 }
 
 // Sums of eight values over a warp by halving: lane l ends with the total of value
@@ -155,6 +157,7 @@ struct CgrShared {
   double keep2;                  // squared growth of the residual up to which the direction is kept
   // the block's lists (CgrPlan's, in shared memory)
   int c0, c1, chunk, nbcap, rcap, nbord, nint, nrem;
+  unsigned polls;         // CgrArgs::polls
   double* wr;             // [chunk][CR_WR] wrenches of the block's contacts (viewed as T)
   double* wl;             // [nbcap][CR_WL] body intermediates (viewed as T)
   double* bw;             // [nbcap][2] 1/m, 1/I of the bodies (viewed as T)
@@ -242,7 +245,7 @@ __device__ __forceinline__ Summed<T> sum_gather(CgrShared& sh, u64* buf, DevCtl*
       }
     }
     if (ok) break;
-    if (give_up(ctl, spins)) {
+    if (give_up(ctl, spins, sh.polls)) {
       fail = 1;
       break;
     }
@@ -592,7 +595,7 @@ __device__ __forceinline__ bool bodies(CgrShared& B, u64* halo, unsigned tag, De
         }
       }
       if (ok) break;
-      if (give_up(ctl, spins)) {
+      if (give_up(ctl, spins, B.polls)) {
         fail = 1;
         break;
       }
@@ -1043,6 +1046,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
     sh.chunk = A.chunk;
     sh.nbcap = A.nbcap;
     sh.rcap = A.rcap;
+    sh.polls = A.polls;
     sh.nbord = A.pl.head[4 * blockIdx.x];
     sh.nint = A.pl.head[4 * blockIdx.x + 1];
     sh.nrem = A.pl.head[4 * blockIdx.x + 2];
@@ -1067,6 +1071,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
     }
     return;
   }
+  if ((int)blockIdx.x == A.absent && A.absent_at == 0) return;
   __syncthreads();
   copy_lists(A.pl, sh);
 
@@ -1102,6 +1107,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_cg_resident(const __grid_constant_
   }
   __syncthreads();
   int iters = 0, repl = 0, status = 0;
+  if ((int)blockIdx.x == A.absent) return;
   if (!(sh.rel <= A.tol)) {
     OWN own;
     own.load(A, sh, s, dinv);
@@ -1287,6 +1293,9 @@ bool launch_cg_resident(qp_ctx* c, const double* rhs, double* dx, double tol, do
   A.inner_tol = inner_tol;
   A.maxit = maxit;
   A.max_outer = max_outer;
+  A.polls = c->cgr_test ? c->cgr_test->polls : CGR_POLLS;
+  A.absent = c->cgr_test ? c->cgr_test->absent : -1;
+  A.absent_at = c->cgr_test ? c->cgr_test->at : 0;
   A.r64 = static_cast<double*>(c->v64[5].ensure((size_t)c->P * sizeof(double)));
   A.xbest = static_cast<double*>(c->v64[6].ensure((size_t)c->P * sizeof(double)));
   const size_t words = 2 * (size_t)G * CR_HALO * A.rcap + 2 * CR_RED;

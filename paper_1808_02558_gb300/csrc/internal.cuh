@@ -54,6 +54,13 @@ struct DevCtl {
 
 enum Scal { S_ETA = 0, S_T, S_RDUAL, S_RT, S_S, S_RELRES, S_BNORM, S_SMAX, S_RCENT, S_TAGS };
 
+// k_cg_resident: polls of a wait (each takes an L2 round trip, at least 400 cycles; about a
+// second), and what the self-test of its waits changes
+constexpr unsigned CGR_POLLS = 4u << 20;
+struct CgrTest {
+  unsigned polls;
+  int absent, at;
+};
 constexpr int CGR_NO_ROOM = 3;  // k_cg_resident: a block's bodies do not fit its shared memory
 
 struct QTTCore;
@@ -114,6 +121,7 @@ struct qp_ctx {
   unsigned cgr_epoch = 0, cgr_last = 0;
   qp_solver solver_used = QP_SOLVER_NONE;  // kernel of the last solve
   int cgr_launches = 0;
+  const qp::CgrTest* cgr_test = nullptr;  // set during qp_selftest_resident
   qp::Buf mp_act, mp_w, mp_grad, mp_sum;  // learned warm start: activations, BF16 weights, scratch
   qp::Buf batch64, batch32, batch_table;  // batched solves: per-scene vectors; table (first context)
   qp::Buf batch_qw, tune_buf;  // batched QTT work buffers; tile-shape probe data

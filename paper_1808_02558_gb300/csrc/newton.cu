@@ -2501,6 +2501,13 @@ static qp_solve_stats solve_stats(qp_ctx* c, const DevCtl& h) {
   return out;
 }
 
+// The blocks of S = N.
+static void zero_schur_blocks(qp_ctx* c) {
+  const size_t n = 6 * (size_t)(c->Nc > 0 ? c->Nc : 1);
+  QP_CUDA(cudaMemsetAsync(c->H.p, 0, n * sizeof(double), c->stream));
+  QP_CUDA(cudaMemsetAsync(c->H32.p, 0, n * sizeof(float), c->stream));
+}
+
 // solve S dx = rhs with the current H blocks (already built for st)
 static qp_solve_stats solve_once(qp_ctx* c, const double* rhs, double* dx, const qp_solve_opts* o) {
   ensure_partial(c);
@@ -3030,8 +3037,7 @@ int newton_solve(qp_ctx_t c, const qp_state* st, const double* rhs, double* dx, 
   check_ready(c, st);
   QP_REQUIRE(rhs && dx && rhs != dx, QP_INVALID_ARG, "newton_solve: null or aliased vectors");
   if (st) launch_schur_blocks(c, st->gamma, st->lambda);
-  else QP_CUDA(cudaMemsetAsync(c->H.p, 0, 6 * (size_t)(c->Nc > 0 ? c->Nc : 1) * sizeof(double), c->stream));
-  if (!st) QP_CUDA(cudaMemsetAsync(c->H32.p, 0, 6 * (size_t)(c->Nc > 0 ? c->Nc : 1) * sizeof(float), c->stream));
+  else zero_schur_blocks(c);
   qp_solve_stats s = solve(c, rhs, dx, o);
   if (stats) *stats = s;
   if (s.status == QP_TIMEOUT) throw Error{QP_TIMEOUT, "newton_solve: device barrier wait expired"};
@@ -3094,6 +3100,30 @@ int qp_selftest_barrier(qp_ctx_t c, long long budget, int absent_block, int* dev
   QP_CUDA(cudaLaunchCooperativeKernel((const void*)k_barrier_probe, dim3(c->num_sms), dim3(128), args, 0, c->stream));
   DevCtl h = read_ctl(c);
   *device_status = h.err;
+  API_END(c)
+}
+
+int qp_selftest_resident(qp_ctx_t c, const double* rhs, double* dx, int mixed, int polls, int absent_block, int at,
+                         int* device_status) {
+  API_BEGIN(c)
+  check_ready(c, nullptr);
+  QP_REQUIRE(rhs && dx && rhs != dx && device_status, QP_INVALID_ARG, "qp_selftest_resident: null or aliased pointers");
+  QP_REQUIRE(polls > 0 && (unsigned)polls <= CGR_POLLS && absent_block < c->num_sms && (at == 0 || at == 1),
+             QP_INVALID_ARG, "qp_selftest_resident: need 0 < polls <= the solver's own, a block or -1, and at 0 or 1");
+  zero_schur_blocks(c);
+  qp_solve_opts o{};
+  o.tol = 1e-2;
+  o.maxit = 1;
+  o.mixed = mixed;
+  const CgrTest test{(unsigned)polls, absent_block, at};
+  c->cgr_test = &test;
+  struct Reset {
+    qp_ctx* c;
+    ~Reset() { c->cgr_test = nullptr; }
+  } reset{c};
+  const qp_solve_stats s = solve_once(c, rhs, dx, &o);
+  QP_REQUIRE(c->solver_used == QP_SOLVER_RESIDENT, QP_INVALID_ARG, "qp_selftest_resident: the contact set is not resident");
+  *device_status = s.status == QP_TIMEOUT ? QP_TIMEOUT : QP_OK;
   API_END(c)
 }
 
