@@ -13,6 +13,7 @@
 #include <mutex>
 
 #include "internal.cuh"
+#include "pair.cuh"
 #include "tc.cuh"
 
 namespace qp {
@@ -454,10 +455,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // in FP64.
 constexpr int WG_CHUNK = 256;
 
-// d = a b + d on pairs of FP32 values
-__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
 __device__ __forceinline__ unsigned long long dup2(float v) {
   unsigned long long d;
   asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));

@@ -19,6 +19,7 @@
 // 484 -> 266 us.
 #pragma once
 
+#include "pair.cuh"
 #include "qtt_dev.cuh"
 
 namespace qp {
@@ -30,9 +31,6 @@ constexpr int QT_MAXM = 5;         // cores a pass at ranks up to 10
 
 typedef unsigned long long u64x;
 
-__device__ __forceinline__ void fma2(u64x& d, u64x a, u64x b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
 __device__ __forceinline__ u64x pack2(float a, float b) {
   u64x d;
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
