@@ -158,11 +158,11 @@ def job_throughput(local_units, local_ms, world):
 
 # ---------------------------------------------------------------------- our arm
 STATUS_NAMES = {0: "ok", -4: "not_converged", -5: "breakdown", -6: "linesearch_fail", -7: "timeout"}
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_pcg<float, void>
-# launch of the 40^3 window (mean of three consecutive launches), from an ncu capture of
-# this kernel version (caches flushed by ncu before each launch).  Reset to None when the
-# kernel changes.
-KPCG_DRAM_BYTES_PER_LAUNCH = 137.2e6
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the kernel that
+# solves the 40^3 window's systems, k_cg_resident<float, Own<float, 2>, 640> (mean of three
+# consecutive launches), from an ncu capture of this kernel version (caches flushed by ncu
+# before each launch).  Reset to None when the kernel changes.
+RESIDENT_DRAM_BYTES_PER_LAUNCH = 127.2e6
 
 
 # FP32 CUDA-core peak of the part from its unit counts: 152 SMs x 128 FP32 lanes x
@@ -170,14 +170,44 @@ KPCG_DRAM_BYTES_PER_LAUNCH = 137.2e6
 FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 
-def qtt_apply_roofline(t, nbytes, flops, passes, d):
+def qtt_schedule(ranks):
+    """Cores per pass of qtt_apply with FP32 vectors, from the last core down (the rules of
+    csrc/qtt_tile.cuh and csrc/qtt_dev.cuh, without the tensor-core steps of dense cores): up
+    to five cores in shared memory (four above rank 10) in equal shares, else two where
+    their ranks are at most 12, else one."""
+    d, k, out = len(ranks) - 1, len(ranks) - 1, []
+    while k >= 1:
+        low, run, most, r = d - k, 0, 5, ranks[k]
+        while k - run >= 1 and r <= 16 and ranks[k - run - 1] <= 16:
+            if max(r, ranks[k - run - 1]) > 10:
+                most = 4
+            r = ranks[k - run - 1]
+            run += 1
+        if low == 0:
+            most = 5
+        groups = -(-run // most)
+        share = 5 if low == 0 else (-(-run // groups) if run else 0)
+        m, r = 0, ranks[k]
+        while m < min(share, run) and d - m - 1 >= 5:
+            r = max(r, ranks[k - m - 1])
+            m += 1
+        if 0 < low < 5 or m < 2 or r > 16 or (low == 0 and k - m > 0 and m < 5) or (r > 12 and m < 4):
+            fuse = k >= 2 and max(ranks[k - 1], ranks[k]) <= 12 and \
+                ranks[k - 1] * ranks[k] + ranks[k - 2] * ranks[k - 1] <= 288
+            m = 2 if fuse else 1
+        out.append(m)
+        k -= m
+    return out
+
+
+def qtt_apply_roofline(t, nbytes, flops, plan):
     """Roofline entry of one QTT apply: HBM-bound when its flop/byte is below the
     ridge of the FP32 ALU peak over the measured HBM peak, ALU-bound above."""
     hbm, src = peaks()[0], peaks()[1]
     ridge = FP32_ALU_TFLOPS * 1e12 / (hbm * 1e9)
     out = {"us": t * 1e6, "bytes": nbytes, "flops": flops, "flop_per_byte": flops / nbytes,
            "ridge_flop_per_byte": ridge, "gbs": nbytes / t / 1e9, "tflops": flops / t / 1e12,
-           "schedule": f"{passes} passes for {d} cores (two cores per pass where ranks <= 12)"}
+           "schedule": f"{len(plan)} passes for {sum(plan)} cores ({'/'.join(map(str, plan))})"}
     if flops / nbytes < ridge:
         out.update({"bound": "hbm", "achieved": nbytes / t / 1e9, "peak": hbm, "unit": "GB/s",
                     "frac": nbytes / t / 1e9 / hbm, "peak_source": src})
@@ -193,6 +223,35 @@ def solve_bytes(Nc, M, nrow, iters, outer):
     inner = iters * (Nc * 100 + M * 48 + 10 * 4 * nrow)
     outer_b = (outer + 1) * (Nc * 200 + M * 96 + 5 * 8 * nrow)
     return inner + outer_b
+
+
+def resident_bytes(Nc, nrow, outer):
+    """Bytes that one mixed solve in the resident kernel has to read and write: records,
+    blocks, diagonal and lists at the start and after each FP64 residual (FP32), and per
+    residual the FP64 records and blocks and five FP64 values a row.  Its iterations move
+    nothing but the sums of bodies on block borders."""
+    start = Nc * (64 + 24 + 16) + 3 * 4 * nrow
+    residual = Nc * (128 + 48) + 5 * 8 * nrow
+    return (outer + 1) * start + outer * residual + 2 * 8 * nrow
+
+
+def solve_roofline(binding, used, Nc, M, iters, outer, ms, workload):
+    """Roofline entry of the kernel that ran the window's solves (`used`)."""
+    peak, src = peaks()
+    nrow = 3 * Nc
+    resident = used == binding.QP_SOLVER_RESIDENT
+    total = sum(resident_bytes(Nc, nrow, ou) if resident else solve_bytes(Nc, M, nrow, it, ou)
+                for it, ou in zip(iters, outer))
+    ach = total / (sum(ms) / 1e3) / 1e9
+    out = {"kernel": "k_cg_resident (Jacobi-CG on chip)" if resident else "k_pcg (persistent PCG)",
+           "bound": "latency" if resident else "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
+           "frac": ach / peak, "peak_source": src, "us_per_iteration": sum(ms) * 1e3 / max(1, sum(iters)),
+           "traffic": RESIDENT_DRAM_BYTES_PER_LAUNCH if resident and workload == "pile40p" else None,
+           "traffic_unit": "bytes per launch (one Newton solve)"}
+    if resident:
+        out["note"] = ("an iteration is one exchange and one sum over the blocks through L2; its vectors and "
+                       "geometry stay in registers and shared memory")
+    return out
 
 
 def run_ours(args):
@@ -271,11 +330,8 @@ def run_ours(args):
     value, total_ms = job_throughput(float(solved), sum(step_ms), world)
     pdip_steps_per_s, _ = job_throughput(float(stepped), sum(step_ms), world)
 
-    # roofline of the dominant kernel (persistent PCG)
-    nrow = 3 * Nc
-    bytes_per = [solve_bytes(Nc, M, nrow, it, ou) for it, ou in zip(iters, outer)]
-    ach = sum(bytes_per) / (sum(pcg_ms) / 1e3) / 1e9
-    peak, src = peaks()
+    # roofline of the dominant kernel (the window's Krylov solves)
+    roof = solve_roofline(binding, ctx.solver_used()[0], Nc, M, iters, outer, pcg_ms, args.workload)
 
     # QTT leg (Sec. 3.3): the same PDIP iterates solved with the QTT-preconditioned
     # PCG, the preconditioner refreshed (compressed + inverted, warm-started) each step
@@ -343,19 +399,14 @@ def run_ours(args):
             e1.record(stream)
             e1.synchronize()
             ap_ms.append(e0.elapsed_time(e1))
-        # schedule of qtt_apply: cores d, d-1, ... in passes of two where both ranks of
-        # the pair and the rank below are <= 12 (else one); a pass reads r_in * N and
-        # writes r_out * N FP32 values.  Flops: core k is applied to N/2 column items,
-        # each a (2 r_{k-1}) x (2 r_k) matrix times a 2 r_k vector, i.e. 4 r_{k-1} r_k
-        # multiply-adds = 8 r_{k-1} r_k flops, so 4 r_{k-1} r_k N flops per core
-        ap_bytes, ap_passes, k = 0, 0, len(ranks) - 1
-        while k >= 1:
-            fuse = k >= 2 and max(ranks[k - 1], ranks[k]) <= 12 and \
-                ranks[k - 1] * ranks[k] + ranks[k - 2] * ranks[k - 1] <= 288
-            nxt = k - 2 if fuse else k - 1
-            ap_bytes += (ranks[k] + ranks[nxt]) * P * 4
-            ap_passes += 1
-            k = nxt
+        # a pass of qtt_apply reads r_in * N and writes r_out * N FP32 values.  Flops: core
+        # k is applied to N/2 column items, each a (2 r_{k-1}) x (2 r_k) matrix times a
+        # 2 r_k vector, i.e. 4 r_{k-1} r_k multiply-adds = 8 r_{k-1} r_k flops, so
+        # 4 r_{k-1} r_k N flops per core
+        ap_plan, ap_bytes, k = qtt_schedule(ranks), 0, len(ranks) - 1
+        for m in ap_plan:
+            ap_bytes += (ranks[k] + ranks[k - m]) * P * 4
+            k -= m
         ap_flops = sum(4 * ranks[k] * ranks[k + 1] * P for k in range(len(ranks) - 1))
         ap_t = statistics.median(ap_ms) / 1e3
         qv = args.window * 1e3 / statistics.mean(q_ms)
@@ -369,7 +420,7 @@ def run_ours(args):
                                                "krylov_iters_per_solve": statistics.mean(r_it),
                                                "jacobi_fallbacks": r_fb,
                                                "note": "refresh at the first PDIP iteration, reused by the others"},
-                   "qtt_apply": qtt_apply_roofline(ap_t, ap_bytes, ap_flops, ap_passes, len(ranks) - 1)}
+                   "qtt_apply": qtt_apply_roofline(ap_t, ap_bytes, ap_flops, ap_plan)}
         for h in (X, S_tt):
             h.free()
         ctxq.close()
@@ -440,10 +491,7 @@ def run_ours(args):
         "krylov_iters_per_solve": statistics.mean(iters), "refinements_per_solve": statistics.mean(outer),
         "max_rel_res": max(relres), "pcg_ms_per_solve": statistics.mean(pcg_ms),
         "qtt_refresh_ms_per_step": statistics.mean(refresh_ms) if qtt else None,
-        "roofline": {"kernel": "k_pcg (persistent PCG)", "bound": "hbm", "achieved": ach, "peak": peak,
-                     "unit": "GB/s", "frac": ach / peak, "peak_source": src,
-                     "traffic": KPCG_DRAM_BYTES_PER_LAUNCH if args.workload == "pile40p" else None,
-                     "traffic_unit": "bytes per launch (one Newton solve)"},
+        "roofline": roof,
         "qtt_pcg": qtt_out,
         "n_apply": apply_out,
         "e2e": {"value": args.window * 1e3 / e2e_ms_max * world, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
