@@ -7,11 +7,14 @@
 // partial sums of bodies shared with other blocks (about 350 of 610 a block on the
 // 40^3 pile) and seven sums leave an SM.
 //
-// What bounds it: the latency of one exchange between neighbouring blocks and of one
-// sum over all blocks an iteration (about 2400 cycles each, a store and a load
-// through L2), and the shared-memory traffic of the body sums.  The classic
-// persistent kernel (three grid barriers and about 45 MB through L2 an iteration)
-// remains for systems that do not fit, for other preconditioners and for BiCGSTAB.
+// What bounds it: latency.  Of 18 800 cycles an iteration of the 40^3 pile takes (1262
+// contacts a block, mixed; clock stamps of one block), the exchange between neighbouring
+// blocks has 4700 and the sum over all blocks 5400, each with the wait for slower blocks
+// (a store and a load through L2 alone are 2400), and the body sums 6400, shared-memory
+// traffic: a block's own 3900, its border's 2500.  The 8^3 pile in FP64 takes 17 700: 3700,
+// 6800 and 3700, and the 64-cycle latency of the FP64 pipe in all of them.  The classic
+// persistent kernel (three grid barriers and about 45 MB through L2 an iteration) remains
+// for systems that do not fit, for other preconditioners and for BiCGSTAB.
 //
 //   p = z + beta p
 //   contact wrenches D_c p_c into shared memory; a body sums its own; the partial
@@ -35,12 +38,12 @@
 // sum that follows exchange k + 1, for which every block has read exchange k.
 // Every wait is bounded (QP_TIMEOUT).
 //
-// Measured, newton_rhs + newton_solve to 1e-12: the 40^3 pile in mixed precision
-// 2.60 -> 1.55 ms (105 iterations of about 9 us in place of 19, and four FP64 residuals
-// of 58 us), the 8^3 pile in FP64 2.13 -> 0.89 ms (91 iterations of 6 us in place of
-// 22).  The pipelined kernel that mid-size systems used (one grid barrier, records
-// through L2, 15 us an iteration on 57 000 contacts) takes 1.4 to 2 times as long as
-// this and is gone.
+// Measured, newton_rhs + newton_solve to 1e-12, against the classic kernel: the 40^3 pile
+// in mixed precision 2.57 -> 1.44 ms (105 iterations of 9.1 us in place of 19, and four
+// FP64 residuals of 57 us), the 8^3 pile in FP64 2.07 -> 0.87 ms (91 iterations of 8.4 us
+// in place of 22).  The pipelined kernel that mid-size systems used (one grid barrier,
+// records through L2, 15 us an iteration on 57 000 contacts, 5.6 here) takes 1.4 to 2
+// times as long as this and is gone.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -179,8 +182,9 @@ struct CgrCount {
 
 // Sums of up to eight values over all threads of all blocks, bit-identical everywhere
 // (fixed trees, blocks in order).  A block's message is 64 bytes (FP64: 128) that
-// every block polls: about 2400 cycles, the latency of a store and a load through L2
-// (slots by value instead, 16 blocks' words in a line, took 10600 for seven values).
+// every block polls: 2400 cycles for a store and a load through L2, 5400 with the sums on
+// both sides and the wait for slower blocks (slots by value instead, 16 blocks' words in
+// a line, took 10600 for seven values).
 //
 // sum_gather, from the warps' partial sums on: the total of value (lane >> 2) in
 // every lane of warp 0; ok = false when a wait expired.  Inlined into the iteration:

@@ -14,9 +14,9 @@
 // shared-memory loads; every quad feeds eight multiply-adds; zero-padded quads need no
 // per-value tests.  Against two cores a launch through global memory (49 to 60 us each
 // at 2^20, rank 10) a pass of five moves 40 % of the bytes: 66 us, of which 26 at the
-// FP32 rate; the FMA pipe is full while a tile is contracted, and idle for the rest
-// (tiles in and out, a last wave of 1024 tiles on 304 blocks).  The whole product:
-// 484 -> 266 us.
+// FP32 rate.  Over a pass of interior ranks the FMA pipe is busy 42 % of the time (ncu):
+// warps queue for it while a tile is contracted, and it idles for the rest (tiles in and
+// out, barriers between steps, 1024 tiles on 304 blocks).  The whole product: 484 -> 266 us.
 #pragma once
 
 #include "pair.cuh"
